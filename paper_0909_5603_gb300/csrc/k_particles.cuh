@@ -738,7 +738,7 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t)
         if (base + kChunk < count) pos_next = stage(base + kChunk + tid, pb ^ 1);
         if (slot < count && (pos < 0 || pos >= I.cap)) atomicOr(I.err, kErrInternal);
         int l[3] = {0, 0, 0}, cc[3] = {0, 0, 0};
-        // deposit inputs; a lane without a particle deposits zero from inside the tile
+        // deposit inputs
         R o[3] = {R(0.5), R(0.5), R(0.5)};
         int l1[3] = {0, 0, 0};
         R disp[3] = {R(0), R(0), R(0)};
@@ -885,9 +885,13 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t)
             cell_new = cn[0] + I.n[0] * (cn[1] + I.n[1] * cn[2]);
         }
 
-        // ---- Esirkepov deposit into the shared J tile, by every lane of the warp.  FP32:
-        // the chunk's per-component scale (see ChunkAcc) from the warps' bounds, after a
-        // barrier that also completes the previous chunk's fold of A into T.
+        // ---- Esirkepov deposit into the shared J tile, by the lanes that hold a particle: in
+        // a tile's last chunk the others would add zeros to one address, which the shared
+        // atomics serialise lane by lane: 32 wavefronts per add of an empty warp, measured
+        // as 263 instead of 568 atomic wavefronts per warp and 4.29 instead of 4.88 ms on
+        // the 128x128x1024 stage with 2 particles per cell.
+        // FP32: the chunk's per-component scale (see ChunkAcc) from the warps' bounds, after
+        // a barrier that also completes the previous chunk's fold of A into T.
         if constexpr (kFixed) {
             // |f_a| (|d_a| + 2^-18): a particle that changes its nodes forms its weight changes
             // from differences of weights, whose rounding (< 2^-19 in the running sums) is
@@ -920,11 +924,15 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t)
                 sc[a] = __frcp_rn(inv[a]);
             }
             // the current follows the computed displacement (see shape_window)
-            deposit_esirkepov<ND, ORD, true, true, LANEWIN, R>(l, o, l1, o1, disp, fx * sc[0], fy * sc[1], fz * sc[2], I.jlo,
-                                                      jlo_y, jd0, jd01, jst, ChunkAcc{sJA});
+            const unsigned lanes = __ballot_sync(0xffffffffu, have);
+            if (have)
+                deposit_esirkepov<ND, ORD, true, true, LANEWIN, R>(lanes, l, o, l1, o1, disp, fx * sc[0], fy * sc[1],
+                                                                   fz * sc[2], I.jlo, jlo_y, jd0, jd01, jst,
+                                                                   ChunkAcc{sJA});
         } else {
-            deposit_esirkepov<ND, ORD, false, false, false, R>(l, o, l1, o1, disp, fx, fy, fz, I.jlo, jlo_y, jd0, jd01,
-                                                        jst, DoubleAcc{sJD});
+            if (have)
+                deposit_esirkepov<ND, ORD, false, false, false, R>(0u, l, o, l1, o1, disp, fx, fy, fz, I.jlo, jlo_y, jd0,
+                                                                   jd01, jst, DoubleAcc{sJD});
         }
 
         // ---- stable ranking of the chunk by bucket: order (warp, lane), one barrier per

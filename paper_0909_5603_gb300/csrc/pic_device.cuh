@@ -434,8 +434,8 @@ __device__ __forceinline__ void esirkepov3d_extra(const R *S0x, const R *DSx, co
     }
 }
 
-// The deposit of one particle; every lane of the warp calls it (a lane without a particle
-// passes f = 0 and a position inside the tile).  In 2D3V (x-z plane) Wx = DSx (S0z +
+// The deposit of one particle, by the lanes of the warp that hold one (`lanes`: their
+// mask, used by the warp vote below).  In 2D3V (x-z plane) Wx = DSx (S0z +
 // DSz/2), Wz = DSz (S0x + DSx/2) and the out-of-plane Jy = f_y' (S0x S0z + DSx S0z / 2 +
 // S0x DSz / 2 + DSx DSz / 3) with f_y' = (q w / dV) v_y; the 2D3V loops skip zero
 // contributions (up to 16 particles per cell contend there).  kNarrow (3D): the window
@@ -447,7 +447,7 @@ __device__ __forceinline__ void esirkepov3d_extra(const R *S0x, const R *DSx, co
 // warp covers ORD + 1 entries along x and y when none of its particles changes its x or y
 // nodes (one vote per warp), ORD + 2 otherwise, and ORD + 2 along z.
 template <int ND, int ORD, bool kDisp, bool kNarrow, bool kLane, typename R, typename Acc>
-__device__ __forceinline__ void deposit_esirkepov(const int l0[3], const R o0[3], const int l1[3], const R o1[3],
+__device__ __forceinline__ void deposit_esirkepov(unsigned lanes, const int l0[3], const R o0[3], const int l1[3], const R o1[3],
                                                   const R disp[3], R fx, R fy, R fz, int jlo, int jlo_y, int jd0,
                                                   int jd01, int jvol, const Acc &acc)
 {
@@ -466,7 +466,7 @@ __device__ __forceinline__ void deposit_esirkepov(const int l0[3], const R o0[3]
                 esirkepov3d_zextra<ORD + 1, W, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
             if (nwx > ORD + 1 || nwy > ORD + 1)
                 esirkepov3d_extra<ORD + 1, W, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
-        } else if (kNarrow && !__any_sync(0xffffffffu, nwx > ORD + 1 || nwy > ORD + 1)) {
+        } else if (kNarrow && !__any_sync(lanes, nwx > ORD + 1 || nwy > ORD + 1)) {
             esirkepov3d<ORD + 1, ORD + 1, W, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
         } else {
             esirkepov3d<W, W, W, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
