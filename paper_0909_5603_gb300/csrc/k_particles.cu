@@ -23,8 +23,8 @@ __global__ void __launch_bounds__(1024) k_scan(Launch L, int mode, int *const *d
 }
 
 // -------------------------------------------------------------------------------------
-// Read-out of the particles in canonical order: per destination tile, the same source
-// walk as the step, into FP64 / int32 staging arrays at the scanned tile offsets.
+// Read-out of the particles of one instance in canonical order: per destination tile, the
+// same source walk as the step, into staging arrays at the scanned tile offsets.
 // -------------------------------------------------------------------------------------
 // read-out staging, values in the storage precision R (widened to FP64 on the host)
 template <typename R>
@@ -37,18 +37,24 @@ struct Stage {
 };
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_readout(Launch L, const int *const *start, Stage<R> out)
+__global__ void __launch_bounds__(256) k_readout(Launch L, const int *const *start, Stage<R> out, int over)
 {
     __shared__ SrcTable S;
-    const int g = blockIdx.x;
-    const int ii = find_instance(L.tile_start, L.ninst, g);
-    const InstDev &I = L.inst[ii];
-    const int t = g - L.tile_start[ii];
+    // the first blocks take the further windows of crowded tiles (listed by the scan)
+    const InstDev &I = L.inst[0];
+    const int win = readout_window(I.cap);
+    int t = (int)blockIdx.x - over, part = 0;
+    if (t < 0) {
+        if ((int)blockIdx.x >= *I.n_over) return;
+        t = I.over[blockIdx.x].x;
+        part = I.over[blockIdx.x].y;
+    }
     const int cur = *I.cur;
     const int tx = t % I.nt[0], ty = (t / I.nt[0]) % I.nt[1], tz = t / (I.nt[0] * I.nt[1]);
-    build_sources(I, cur, tx, ty, tz, S);
-    const int dst0 = start[ii][t];
-    for (int p = threadIdx.x; p < S.count; p += blockDim.x) {
+    const int dst0 = start[0][t];
+    const int p0 = part * win, p1 = min(start[0][t + 1] - dst0, p0 + win);
+    build_sources(I, cur, tx, ty, tz, p0, p1, S);
+    for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
         const int pos = slot_position(I, cur, S, p);
         if (pos < 0 || pos >= I.cap) { atomicOr(I.err, kErrInternal); continue; }
         const long long q = dst0 + p;
@@ -244,15 +250,16 @@ cudaError_t launch_scan(const Launch &L, int mode, int *const *dst, cudaStream_t
     return cudaGetLastError();
 }
 
-cudaError_t launch_readout(int fp64, const Launch &L, const int *const *start, int *cell, void *off, void *u, void *w,
-                           int *id, cudaStream_t s)
+cudaError_t launch_readout(int fp64, const Launch &L, int cap, const int *const *start, int *cell, void *off, void *u,
+                           void *w, int *id, cudaStream_t s)
 {
+    const int over = cap / readout_window(cap);
     if (fp64) {
         Stage<double> st{cell, (double *)off, (double *)u, (double *)w, id};
-        k_readout<double><<<L.total_tiles, 256, 0, s>>>(L, start, st);
+        k_readout<double><<<L.total_tiles + over, 256, 0, s>>>(L, start, st, over);
     } else {
         Stage<float> st{cell, (float *)off, (float *)u, (float *)w, id};
-        k_readout<float><<<L.total_tiles, 256, 0, s>>>(L, start, st);
+        k_readout<float><<<L.total_tiles + over, 256, 0, s>>>(L, start, st, over);
     }
     return cudaGetLastError();
 }

@@ -18,7 +18,7 @@ static cudaError_t launch_particles_t(const Launch *L, const InstDev *one, size_
         return e == cudaSuccess ? cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : e;
     }
     if (one && L->ninst == 1)
-        k1<<<L->total_tiles, kNT, smem, s>>>(*one);
+        k1<<<L->total_tiles + one->over_max, kNT, smem, s>>>(*one);
     else
         k<<<L->total_tiles, kNT, smem, s>>>(*L);
     return cudaGetLastError();

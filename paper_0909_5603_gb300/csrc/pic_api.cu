@@ -471,8 +471,10 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
     c->d_pencil = (long long *)dalloc(c, 8 * sizeof(long long));
     h.ion_face = dalloc(c, sizeof(double) * (size_t)c->n[2]);
     h.srcrec = (int *)dalloc(c, sizeof(int) * (size_t)h.ntiles * kSrcRec);
+    // parts of crowded tiles: the list, its parts' totals, two ints per tile, the count
+    int *parts = (int *)dalloc(c, sizeof(int) * ((size_t)(2 + kBuckets) * kMaxOver + 2 * (size_t)h.ntiles + 1));
     if (!F || !small || !tiles || !tm || !c->d_inst || !c->d_tile_start || !c->d_cell_start || !c->d_dense || !c->d_sums ||
-        !c->d_start || !c->d_start_ptr || !c->d_pencil || !h.ion_face || !h.srcrec) {
+        !c->d_start || !c->d_start_ptr || !c->d_pencil || !h.ion_face || !h.srcrec || !parts) {
         dfree_all(c);
         delete c;
         return fail(nullptr, PIC_ERR_OOM, "device allocation failed (%zu bytes of fields)", fbytes);
@@ -485,6 +487,11 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
         h.E2[a] = F + (size_t)(12 + a) * h.cstride * c->es;
         h.B2[a] = F + (size_t)(15 + a) * h.cstride * c->es;
     }
+    h.over = (int2 *)parts;
+    h.part_tot = parts + 2 * kMaxOver;
+    h.split = h.part_tot + kBuckets * kMaxOver;
+    h.done = h.split + h.ntiles;
+    h.n_over = h.done + h.ntiles;
     h.cur = small;
     h.err = small + 1;
     h.live = small + 2;
@@ -551,6 +558,8 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
     const long long cstart[2] = {0, c->ncell};
     int *dptr_start = c->d_start;
     bool okc = cudaMemsetAsync(F, 0, fbytes, c->stream) == cudaSuccess && cudaMemsetAsync(small, 0, 4096, c->stream) == cudaSuccess &&
+               cudaMemsetAsync(parts, 0, sizeof(int) * ((size_t)(2 + kBuckets) * kMaxOver + 2 * (size_t)h.ntiles + 1), c->stream) ==
+                   cudaSuccess &&
                cudaMemsetAsync(tiles, 0, sizeof(int) * (size_t)(4 * nt1 + 2 * h.ntiles * kBuckets + h.ntiles), c->stream) == cudaSuccess &&
                cudaMemcpyAsync(tm, maps, sizeof(maps), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
                cudaMemcpyAsync(c->d_tile_start, tstart, sizeof(tstart), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
@@ -759,6 +768,13 @@ static pic_status upload_layout(pic_ctx *c, const std::vector<int> &seg)
         pop[t] = m;
     }
     const int nchunks = cbase[h.ntiles];
+    // Room for parts of crowded tiles (part_chunks) when a tile holds three quarters of the
+    // chunks from which it is split; otherwise none, as idle blocks ahead of the tiles cost
+    // 2 to 23 us a launch (64^3 cells with 16 particles each: 645 against 668 us).  The
+    // chunks the buffers hold bound the parts.
+    int most = 0;
+    for (int t = 0; t < h.ntiles; ++t) most = std::max(most, cbase[t + 1] - cbase[t]);
+    h.over_max = 2 * most > 3 * part_chunks(nchunks) ? std::min(h.chunk_cap / kMinPart, kMaxOver) : 0;
     if (nchunks > h.chunk_cap) return fail(c, PIC_ERR_INTERNAL, "chunk capacity");
     std::vector<int> pre((size_t)std::max(nchunks, 1) * kPre, 0), cbv((size_t)std::max(nchunks, 1) * kBuckets, 0);
     for (int t = 0; t < h.ntiles; ++t) {
@@ -1599,7 +1615,7 @@ static pic_status get_particles_internal(pic_ctx *ctx, int32_t *cell, void *off3
     if (live > cap) return fail(ctx, PIC_ERR_ARG, "cap %lld < %d live particles", (long long)cap, live);
     if (live == 0) return PIC_OK;
     if ((st = ensure_staging(ctx)) != PIC_OK) return st;
-    CUDA_OR_FAIL(ctx, launch_readout(ctx->fp64, ctx->L, ctx->d_start_ptr, ctx->st_cell, ctx->st_off, ctx->st_u, ctx->st_w,
+    CUDA_OR_FAIL(ctx, launch_readout(ctx->fp64, ctx->L, ctx->h.cap, ctx->d_start_ptr, ctx->st_cell, ctx->st_off, ctx->st_u, ctx->st_w,
                                      ctx->st_id, ctx->stream));
     // values copied in the storage precision (FP32: half the bytes) into the caller's
     // arrays, then widened there in place when FP64 values are asked for
@@ -1737,7 +1753,7 @@ static pic_status stage_particles(pic_ctx *c, std::vector<int32_t> &cells, int &
     cells.resize((size_t)std::max(live, 1));
     if (live == 0) return PIC_OK;
     if ((st = ensure_staging(c)) != PIC_OK) return st;
-    CUDA_OR_FAIL(c, launch_readout(c->fp64, c->L, c->d_start_ptr, c->st_cell, c->st_off, c->st_u, c->st_w, c->st_id,
+    CUDA_OR_FAIL(c, launch_readout(c->fp64, c->L, c->h.cap, c->d_start_ptr, c->st_cell, c->st_off, c->st_u, c->st_w, c->st_id,
                                    c->stream));
     CUDA_OR_FAIL(c, cudaMemcpyAsync(cells.data(), c->st_cell, sizeof(int) * (size_t)live, cudaMemcpyDeviceToHost, c->stream));
     CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));

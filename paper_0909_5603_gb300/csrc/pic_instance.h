@@ -27,6 +27,31 @@ constexpr int kRecSlot = 4;                            // sub_slot[kSubCache + 1
 constexpr int kRecPos = kRecSlot + kSubCache + 1;      // sub_pos[kSubCache] from here
 constexpr int kSrcRec = (kRecPos + kSubCache + 3) / 4 * 4;  // ints per tile
 
+// A tile crowded with particles is worked on by several CTAs (parts) of the particle
+// kernel in a launch of one instance.  A part takes part_chunks() chunks; a tile is split
+// when it holds more than twice that.  kMaxOver bounds the parts beyond the first over all
+// tiles: their number is at most total / part_chunks(total) <= kMaxOver = two for each of
+// the 2 x 152 CTAs that are resident, so that the largest part is about half of a CTA's
+// share of the launch: a bunch of 2^20 electrons in 64x64x256 cells, whose fullest tile
+// holds 520 of its 4,500 chunks, is then balanced.  Parts below 8 chunks would spend more on
+// staging the fields and flushing J than on their particles.
+constexpr int kMaxOver = 608;
+constexpr int kMinPart = 8;
+
+__host__ __device__ __forceinline__ int part_chunks(int total_chunks)
+{
+    const int m = (total_chunks + kMaxOver - 1) / kMaxOver;
+    return m > kMinPart ? m : kMinPart;
+}
+
+// Output slots per CTA of the canonical read-out for a buffer of cap particles: a fuller
+// tile is read out by several CTAs (at most cap / window <= 512 beyond the tiles' own).
+__host__ __device__ __forceinline__ int readout_window(int cap)
+{
+    const int w = (cap + 511) / 512;
+    return w > 8192 ? w : 8192;
+}
+
 // Division of 0 <= x < 2^31 by a fixed divisor d >= 1 without a divide instruction
 // (Granlund & Montgomery, "Division by invariant integers using multiplication", 1994,
 // round-up variant): s = ceil(log2 d), m = floor(2^(32+s) / d) + 1 (33 bits), then
@@ -116,6 +141,14 @@ struct InstDev {
     int *tot[2];        // [ntiles * kBuckets] bucket totals of each tile
     int *pop;           // [ntiles] particles in each tile at the step boundary
     int *srcrec;        // [ntiles * kSrcRec] source records of the coming particle phase
+    int *split;         // [ntiles] of the coming particle phase: -1, or, for a tile worked on
+                        // in parts, its first entry in over
+    int *done;          // [ntiles] parts of the tile completed
+    int *n_over;        // entries in over
+    int over_max;       // room in over for the parts of a step: 0 when no tile was near
+                        // crowded at the load, and then no tile is split
+    int2 *over;         // [kMaxOver] (tile, part) of the parts beyond a tile's first
+    int *part_tot;      // [kMaxOver * kBuckets] bucket totals of those parts
     int *cur;           // device parity: which layout/buffer holds the current state
     int *jsel;          // which J array (0: J, 1: Jt) holds the filtered current
     int *err;           // sticky error word

@@ -84,7 +84,8 @@ cudaError_t launch_scan(const Launch &L, int mode, int *const *dst, cudaStream_t
 // per-tile source records of the coming particle phase (after the scan of mode 0)
 cudaError_t launch_tile_sources(const Launch &L, cudaStream_t s);
 // off, u, w: staging in the storage precision (double or float)
-cudaError_t launch_readout(int fp64, const Launch &L, const int *const *start, int *cell, void *off, void *u,
+// cap: the particles its buffers hold
+cudaError_t launch_readout(int fp64, const Launch &L, int cap, const int *const *start, int *cell, void *off, void *u,
                            void *w, int *id, cudaStream_t s);
 cudaError_t launch_particle_sums(int fp64, const Launch &L, double *sums, cudaStream_t s);
 cudaError_t launch_rho(int order, int fp64, const Launch &L, double *rho, cudaStream_t s);

@@ -1,6 +1,6 @@
 """The particle phase over tile populations at the edges of a chunk of 256 particles (a
 warp, a chunk, several chunks, each with a remainder): one crowded tile next to empty
-ones, against the FP64 oracle, for one instance and for a batch.  FP32 after one phase:
+ones, and tiles crowded enough to be worked on in parts by several CTAs, against the FP64 oracle, for one instance and for a batch.  FP32 after one phase:
 J normwise within 2e-6, the bar of the block-scaled accumulation; FP64: 1e-12."""
 import numpy as np
 import pytest
@@ -85,3 +85,23 @@ def test_populations_around_a_chunk(ndim, order, prec, count):
     batch.synchronize()
     for m, o in zip(members, oracles):
         check(m, o, prec, ndim)
+
+
+@pytest.mark.parametrize("count", [16 * 256, 16 * 256 + 1, 24 * 256, 9000])
+@pytest.mark.parametrize("ndim,order,prec", [(3, 2, FP32), (2, 2, FP32), (3, 1, FP64), (2, 2, FP64)])
+def test_crowded_tile_in_parts(ndim, order, prec, count):
+    """A tile of 16 chunks (the most that one CTA takes whole here), one particle more, and
+    further multiples of a part: three phases keep the canonical order (FP64: bit for bit),
+    which the next phase and the read-out find through the parts' joined chunk records."""
+    n, ts = GRID[ndim]
+    fields = synth.smooth_fields(n, ndim, 0.2, seed=22)
+    p = crowd(ndim, count, 300 + count)
+    o = oracle.Sim(ndim, n, (0, 0, 0), (1.0, 1.0, 1.0), DT, order=order, tile=(ts, ts if ndim == 3 else 1, ts))
+    for c, f in enumerate(fields):
+        o.set_field(c, f)
+    o.set_particles(p["cell"], p["off"], p["u"], p["w"], p["id"])
+    g = make(ndim, order, prec, p, fields)
+    for _ in range(3):
+        g.run_phases(pic.PIC_PHASE_PARTICLES)
+        o.particle_phase()
+        check(g, o, prec, ndim)
