@@ -183,9 +183,12 @@ static __device__ void build_sources(const InstDev &I, int lay, int tx, int ty, 
         const int a = max(s0 - (pc - cnt), 0), b = min(s1 - (pc - cnt), cnt);
         int k0 = 0, len = 0;
         if (lane < n && b > a) {
-            const int *tile_cb = cb + (long long)c0 * kBuckets;
-            k0 = chunk_of(tile_cb, nch, d, a);
-            len = chunk_of(tile_cb, nch, d, b - 1) - k0 + 1;
+            len = nch;
+            if (a > 0 || b < cnt) {  // (a whole source needs no search through its records)
+                const int *tile_cb = cb + (long long)c0 * kBuckets;
+                k0 = chunk_of(tile_cb, nch, d, a);
+                len = chunk_of(tile_cb, nch, d, b - 1) - k0 + 1;
+            }
         }
         int pn = len;
 #pragma unroll
