@@ -92,21 +92,22 @@ __global__ void __launch_bounds__(256) k_bhalf(Launch L, int damp)
     Bz[p] = bz;
 }
 
-// The fused Yee update, one CTA per tile and z chunk (maxwell_fused_block).
+// The fused Yee update, one CTA per tile and z chunk (maxwell_fused_block).  The CTA of an
+// instance that finishes last switches it to the buffer pair it wrote (every CTA has read
+// the parity by then), so that no launch follows for it.
 template <typename R, int ND>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_maxwell_fused(Launch L, const long long *tile_start,
-                                                                              int filtered)
+__global__ void __launch_bounds__(MxTile<ND>::X * MxTile<ND>::Y, mx_resident<R, ND>())
+    k_maxwell_fused(Launch L, const long long *tile_start, int filtered)
 {
-    maxwell_fused_block<R, ND>(L, tile_start, filtered, blockIdx.x);
-}
-
-// After the fused update: every instance of the launch switches to the buffer pair it
-// wrote.
-__global__ void k_flip_fields(Launch L)
-{
-    for (int i = threadIdx.x; i < L.ninst; i += blockDim.x) {
-        int *f = L.inst[i].fpar;
-        *f ^= 1;
+    maxwell_fused_block<R, ND, MxTile<ND>::X, MxTile<ND>::Y>(L, tile_start, filtered, blockIdx.x, 0, true);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const int ii = find_instance_ll(tile_start, L.ninst, blockIdx.x);
+        const InstDev &I = L.inst[ii];
+        if (atomicAdd(I.mx_done, 1) == (int)(tile_start[ii + 1] - tile_start[ii]) - 1) {
+            *I.mx_done = 0;
+            *I.fpar ^= 1;
+        }
     }
 }
 
@@ -405,7 +406,14 @@ template <typename R, int ND>
 static cudaError_t maxwell_fused_attr()
 {
     return cudaFuncSetAttribute(k_maxwell_fused<R, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)maxwell_fused_smem<R, ND>());
+                                (int)maxwell_fused_smem<R, ND, MxTile<ND>::X, MxTile<ND>::Y>());
+}
+
+template <typename R, int ND>
+static void maxwell_fused_t(const Launch &L, const long long *tile_start, unsigned nb, int filtered, cudaStream_t s)
+{
+    constexpr int X = MxTile<ND>::X, Y = MxTile<ND>::Y;
+    k_maxwell_fused<R, ND><<<nb, X * Y, maxwell_fused_smem<R, ND, X, Y>(), s>>>(L, tile_start, filtered);
 }
 
 cudaError_t launch_maxwell_fused(int fp64, int ndim, const Launch &L, const long long *tile_start, long long ntiles,
@@ -413,14 +421,12 @@ cudaError_t launch_maxwell_fused(int fp64, int ndim, const Launch &L, const long
 {
     if (ntiles <= 0) return cudaSuccess;
     const unsigned nb = (unsigned)ntiles;
-    if (fp64) {
-        if (ndim == 3) k_maxwell_fused<double, 3><<<nb, 256, maxwell_fused_smem<double, 3>(), s>>>(L, tile_start, filtered);
-        else k_maxwell_fused<double, 2><<<nb, 256, maxwell_fused_smem<double, 2>(), s>>>(L, tile_start, filtered);
-    } else {
-        if (ndim == 3) k_maxwell_fused<float, 3><<<nb, 256, maxwell_fused_smem<float, 3>(), s>>>(L, tile_start, filtered);
-        else k_maxwell_fused<float, 2><<<nb, 256, maxwell_fused_smem<float, 2>(), s>>>(L, tile_start, filtered);
-    }
-    k_flip_fields<<<1, 128, 0, s>>>(L);
+    if (fp64)
+        ndim == 3 ? maxwell_fused_t<double, 3>(L, tile_start, nb, filtered, s)
+                  : maxwell_fused_t<double, 2>(L, tile_start, nb, filtered, s);
+    else
+        ndim == 3 ? maxwell_fused_t<float, 3>(L, tile_start, nb, filtered, s)
+                  : maxwell_fused_t<float, 2>(L, tile_start, nb, filtered, s);
     return cudaGetLastError();
 }
 

@@ -60,9 +60,12 @@ __device__ __forceinline__ R damp_factor(const InstDev &I, const CellPos &c)
 // step, damped B half step.  It reads E^n, B^n and J once and writes E^{n+1}, B^{n+1}
 // once (60 bytes per cell in FP32 instead of 120 for the three-kernel sequence).  The
 // inputs are the current E / B buffer pair and the outputs go to the other one (*fpar
-// flips after the kernel), so no CTA overwrites a value that a neighbouring CTA still
-// reads.  A CTA takes an x-y tile of TX x TY columns (one thread each) and marches
-// along z through a chunk of TZ planes, keeping in shared memory E^n of three planes on
+// flips after the last CTA), so no CTA overwrites a value that a neighbouring CTA still
+// reads.  A cell near a periodic face is also stored at its images in the ghost layers
+// beyond the opposite faces (what the gather's TMA boxes read there), instead of one ghost
+// copy launch per periodic axis.  A CTA takes an x-y tile of TX x TY columns (one thread
+// each) and marches
+// along z through a chunk of tz planes, keeping in shared memory E^n of three planes on
 // the tile widened by [-1, +2] in x and y, B^{n+1/2} of three planes on [-1, +1] and
 // E^{n+1} of two planes on [0, +1].  For the output plane k, between two barriers:
 //   B^{n+1/2}(k+2) = B^n - dt/2 curl E^n        (E^n of planes k+2, k+3)
@@ -72,22 +75,10 @@ __device__ __forceinline__ R damp_factor(const InstDev &I, const CellPos &c)
 // with the loads of the next plane issued one plane ahead.  Outside an absorbing box
 // every field is zero; periodic axes wrap.  Each value is formed by the same expression
 // as in k_bhalf / k_efull; the in-plane offsets of a thread's cells are computed once.
-template <int ND>
-struct MxTile;
-template <>
-struct MxTile<3> {
-    static constexpr int X = 32, Y = 8, Z = 32;
-};
-template <>
-struct MxTile<2> {
-    static constexpr int X = 256, Y = 1, Z = 32;
-};
-
-template <typename R, int ND>
+template <typename R, int ND, int X, int Y>
 constexpr size_t maxwell_fused_smem()
 {
     constexpr int HY = ND == 3 ? 1 : 0;
-    constexpr int X = MxTile<ND>::X, Y = MxTile<ND>::Y;
     constexpr size_t NE = (size_t)(X + 3) * (Y + 3 * HY), NB = (size_t)(X + 2) * (Y + 2 * HY), NQ = (size_t)(X + 1) * (Y + HY);
     return sizeof(R) * 3 * (3 * NE + 3 * NB + 2 * NQ);
 }
@@ -105,16 +96,19 @@ __device__ __forceinline__ bool mx_axis(int q, int n, int bc, int &w)
     return true;
 }
 
-template <typename R, int ND>
+// Block g of the launch's tiles (tile_start: the instances' first tiles), by TX x TY threads.
+// tz: planes per chunk (0: the instance's own, mx_planes).  images: also store the periodic
+// images of the cells.
+template <typename R, int ND, int TX, int TY>
 __device__ __forceinline__ void maxwell_fused_block(const Launch &L, const long long *tile_start, int filtered,
-                                                    const long long g)
+                                                    const long long g, int tz, bool images)
 {
-    constexpr int TX = MxTile<ND>::X, TY = MxTile<ND>::Y, TZ = MxTile<ND>::Z;
+    constexpr int NT = TX * TY;
     constexpr int HY = ND == 3 ? 1 : 0;
     constexpr int EX = TX + 3, NE = EX * (TY + 3 * HY);  // E^n region: [-1, +2]
     constexpr int BX = TX + 2, NB = BX * (TY + 2 * HY);  // B^{n+1/2} region: [-1, +1]
     constexpr int QX = TX + 1, NQ = QX * (TY + HY);      // E^{n+1} region: [0, +1]
-    static_assert(TX * TY == 256 && NE <= 512 && NB <= 512 && NQ <= 512, "two region cells per thread");
+    static_assert(NE <= 2 * NT && NB <= 2 * NT && NQ <= 2 * NT, "two region cells per thread");
     extern __shared__ __align__(16) unsigned char msm[];
     R *sE = (R *)msm;     // [3 planes][3 comps][NE]
     R *sH = sE + 9 * NE;  // [3][3][NB]
@@ -128,8 +122,9 @@ __device__ __forceinline__ void maxwell_fused_block(const Launch &L, const long 
     const int x0 = (int)(r % ntx) * TX;
     r /= ntx;
     const int y0 = (int)(r % nty) * TY;
-    const int z0 = (int)(r / nty) * TZ;
-    const int z1 = min(z0 + TZ, n2);
+    if (tz == 0) tz = I.mx_planes;
+    const int z0 = (int)(r / nty) * tz;
+    const int z1 = min(z0 + tz, n2);
     const int par = *(volatile const int *)I.fpar;
     // the components of each field are cstride elements apart
     const long long cs = I.cstride;
@@ -159,13 +154,18 @@ __device__ __forceinline__ void maxwell_fused_block(const Launch &L, const long 
     R qf[2], tf, unused;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-        const int e = tid + 256 * j, b = tid + 256 * j, q = tid + 256 * j;
+        const int e = tid + NT * j, b = tid + NT * j, q = tid + NT * j;
         eok[j] = e < NE && inplane(e % EX - 1, e / EX - HY, eoff[j], unused);
         bok[j] = b < NB && inplane(b % BX - 1, b / BX - HY, boff[j], unused);
         qok[j] = q < NQ && inplane(q % QX, q / QX, qoff[j], qf[j]);
     }
     const int tx = tid % TX, ty = tid / TX;
     tok = x0 + tx < n0 && y0 + ty < n1 && inplane(tx, ty, toff, tf);
+    // the images of this column in the ghost layers of periodic axes: bit 0 (1) of mx when x
+    // is within the ghost width of the lower (upper) face, my for y
+    const int mx = images && I.bc[0] == 0 ? (x0 + tx < I.gh[0] ? 1 : 0) | (x0 + tx >= n0 - I.gh[0] ? 2 : 0) : 0;
+    const int my = ND == 3 && images && I.bc[1] == 0 ? (y0 + ty < I.gh[1] ? 1 : 0) | (y0 + ty >= n1 - I.gh[1] ? 2 : 0) : 0;
+    const bool zimg = images && I.bc[2] == 0;
     // z: padded plane offset of plane k, false outside an absorbing box
     auto zplane = [&](int k, long long &zo, R &fz) -> bool {
         int z;
@@ -189,9 +189,9 @@ __device__ __forceinline__ void maxwell_fused_block(const Launch &L, const long 
         R *d = sE + slot3(k) * 3 * NE;
 #pragma unroll
         for (int j = 0; j < 2; ++j)
-            if (tid + 256 * j < NE)
+            if (tid + NT * j < NE)
 #pragma unroll
-                for (int c = 0; c < 3; ++c) d[c * NE + tid + 256 * j] = v[j][c];
+                for (int c = 0; c < 3; ++c) d[c * NE + tid + NT * j] = v[j][c];
     };
     // B^{n+1/2}(k) from E^n of planes k, k+1 and B^n(k) (bv)
     auto makeH = [&](int k, const R (&bv)[2][3]) {
@@ -202,7 +202,7 @@ __device__ __forceinline__ void maxwell_fused_block(const Launch &L, const long 
         R *H = sH + slot3(k) * 3 * NB;
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const int b = tid + 256 * j;
+            const int b = tid + NT * j;
             if (b >= NB) continue;
             R hb[3] = {R(0), R(0), R(0)};
             if (zk && bok[j]) {
@@ -235,7 +235,7 @@ __device__ __forceinline__ void maxwell_fused_block(const Launch &L, const long 
         R *Q = sQ + (k & 1) * 3 * NQ;
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const int q = tid + 256 * j;
+            const int q = tid + NT * j;
             if (q >= NQ) continue;
             R en[3] = {R(0), R(0), R(0)};
             if (zk && qok[j]) {
@@ -291,6 +291,24 @@ __device__ __forceinline__ void maxwell_fused_block(const Launch &L, const long 
         Eout[p] = ex;
         Eout[cs + p] = ey;
         Eout[2 * cs + p] = ez;
+        const int mz = zimg ? (k < I.gh[2] ? 1 : 0) | (k >= n2 - I.gh[2] ? 2 : 0) : 0;
+        if (mx | my | mz) {
+            // every combination of staying (0), + n (1) and - n (2) along the three axes
+#pragma unroll 1
+            for (int m = 1; m < 27; ++m) {
+                const int ax = m % 3, ay = (m / 3) % 3, az = m / 9;
+                if ((ax && !(mx & ax)) || (ay && !(my & ay)) || (az && !(mz & az))) continue;
+                const long long s = p + (ax == 1 ? n0 : ax == 2 ? -n0 : 0) +
+                                    I.sy * (long long)(ay == 1 ? n1 : ay == 2 ? -n1 : 0) +
+                                    I.sz * (long long)(az == 1 ? n2 : az == 2 ? -n2 : 0);
+                Bout[s] = bx;
+                Bout[cs + s] = by;
+                Bout[2 * cs + s] = bz;
+                Eout[s] = ex;
+                Eout[cs + s] = ey;
+                Eout[2 * cs + s] = ez;
+            }
+        }
     };
 
     R vE[2][3], cB[2][3], cJ[2][3], nB[2][3], nJ[2][3];

@@ -93,10 +93,16 @@ __device__ __noinline__ void particle_item(const Launch &L, int g)
     particle_tile_of_launch<ND, ORD, float, 0, false>(L, g);
 }
 
+constexpr int kPersistPlanes = 32;  // planes of a fused Yee item
+template <int ND>
+struct PersistMx {  // columns of a fused Yee item, one per thread of the CTA
+    static constexpr int X = ND == 3 ? 32 : kNT, Y = ND == 3 ? 8 : 1;
+};
+
 template <int ND>
 __device__ __noinline__ void maxwell_item(const Launch &L, const long long *mx_start, int filtered, long long g)
 {
-    maxwell_fused_block<float, ND>(L, mx_start, filtered, g);
+    maxwell_fused_block<float, ND, PersistMx<ND>::X, PersistMx<ND>::Y>(L, mx_start, filtered, g, kPersistPlanes, false);
 }
 
 __device__ __noinline__ void filter_any(const Launch &L, const long long *pen, int axis, int src_is_jt, long long g,
@@ -267,7 +273,8 @@ size_t persist_smem(int ndim, size_t particle_smem)
 {
     // the particle phase's dynamic shared memory, or the largest scratch of another phase
     size_t m = particle_smem;
-    m = std::max(m, ndim == 3 ? maxwell_fused_smem<float, 3>() : maxwell_fused_smem<float, 2>());
+    m = std::max(m, ndim == 3 ? maxwell_fused_smem<float, 3, PersistMx<3>::X, PersistMx<3>::Y>()
+                              : maxwell_fused_smem<float, 2, PersistMx<2>::X, PersistMx<2>::Y>());
     m = std::max(m, sizeof(float) * 8 * 3 * (size_t)(kPencil + 2 * 4) + 128);
     m = std::max(m, sizeof(SrcScratch) * 8 + 128);
     m = std::max(m, sizeof(int) * 66 + 128);
@@ -282,7 +289,7 @@ cudaError_t persist_blocks_per_sm(int ndim, int order, size_t smem, int *bps)
 PersistPlan::PersistPlan() : impl(new Impl) {}
 PersistPlan::~PersistPlan() { delete impl; }
 
-cudaError_t PersistPlan::build(const std::vector<PersistCounts> &inst, void *(*alloc)(void *, size_t), void *user)
+cudaError_t PersistPlan::build(int ndim, const std::vector<PersistCounts> &inst, void *(*alloc)(void *, size_t), void *user)
 {
     const int n = (int)inst.size();
     impl->ninst = n;
@@ -298,7 +305,10 @@ cudaError_t PersistPlan::build(const std::vector<PersistCounts> &inst, void *(*a
             case kPhSources: c = (k.ntiles + 7) / 8; break;
             case kPhParticles: c = k.ntiles; break;
             case kPhFilterX: case kPhFilterY: case kPhFilterZ: c = k.pencils[p - kPhFilterX]; break;
-            case kPhMaxwell: c = k.mx_tiles; break;
+            case kPhMaxwell:
+                c = ndim == 3 ? maxwell_tiles(k.n, PersistMx<3>::X, PersistMx<3>::Y, kPersistPlanes)
+                              : maxwell_tiles(k.n, PersistMx<2>::X, PersistMx<2>::Y, kPersistPlanes);
+                break;
             case kPhGhostX: case kPhGhostY: case kPhGhostZ: c = (k.ghost[p - kPhGhostX] + kGhostElems - 1) / kGhostElems; break;
             default: c = 1;
             }
@@ -319,8 +329,8 @@ cudaError_t PersistPlan::build(const std::vector<PersistCounts> &inst, void *(*a
 long long PersistPlan::items_per_step() const { return impl->per_step; }
 
 cudaError_t PersistPlan::launch(const Launch &L, int ndim, int order, int nsteps, int passes, int filtered,
-                                const long long *pencil_tables, const long long *mx_start, size_t smem, int grid,
-                                long long spin_limit, int stall_inst, cudaStream_t s)
+                                const long long *pencil_tables, size_t smem, int grid, long long spin_limit,
+                                int stall_inst, cudaStream_t s)
 {
     cudaError_t e = cudaMemsetAsync(impl->d_counters, 0, impl->counter_bytes, s);
     if (e != cudaSuccess) return e;
@@ -333,7 +343,7 @@ cudaError_t PersistPlan::launch(const Launch &L, int ndim, int order, int nsteps
     for (int p = 0; p <= kPhCount; ++p) D.phase_base[p] = impl->phase_base[p];
     D.pre = impl->d_pre;
     for (int a = 0; a < 3; ++a) D.pencil[a] = pencil_tables + (size_t)a * (impl->ninst + 1);
-    D.mx_start = mx_start;
+    D.mx_start = impl->d_pre + (size_t)kPhMaxwell * (impl->ninst + 1);
     D.cursor = impl->d_counters;
     D.abort_flag = (int *)(impl->d_counters + 1);
     D.done = (int *)(impl->d_counters + 2);

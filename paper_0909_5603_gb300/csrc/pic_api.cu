@@ -499,6 +499,8 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
     h.lost = (unsigned long long *)(small + 4);
     h.phase = small + 6;
     h.fpar = small + 8;
+    h.mx_done = small + 9;
+    h.mx_planes = maxwell_planes(&c->n, 1, c->ndim, c->fp64);
     h.seg[0] = tiles;
     h.seg[1] = tiles + nt1;
     h.chunk_base[0] = tiles + 2 * nt1;
@@ -550,7 +552,7 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
     }
     long long pencils[8];
     for (int a = 0; a < 4; ++a) {
-        c->pencil_total[a] = a == 3 ? maxwell_tiles(c->n, c->ndim) : o.filter_passes > 0 ? filter_pencils(c->n, c->ndim, a) : 0;
+        c->pencil_total[a] = a == 3 ? maxwell_tiles(c->n, c->ndim, h.mx_planes) : o.filter_passes > 0 ? filter_pencils(c->n, c->ndim, a) : 0;
         pencils[2 * a] = 0;
         pencils[2 * a + 1] = c->pencil_total[a];
     }
@@ -1299,16 +1301,18 @@ static pic_status enqueue_step(pic_ctx *c, int mask)
     }
     if (mask & PIC_PHASE_MAXWELL) {
         tm.begin(3);
+        bool fused = false;
         std::vector<pic_ctx *> ants;  // instances with a laser antenna
         if (c->ant_on) ants.push_back(c);
         for (auto m : c->members)
             if (m->ant_on) ants.push_back(m);
         if (ants.empty() && c->opt.solver == PIC_SOLVER_YEE && c->pencil_total[3] > 0) {
-            // the fused update: one launch, then the buffer switch
+            // the fused update, with the buffer switch and the periodic images
             const int nin = c->is_batch ? (int)c->members.size() : 1;
             CUDA_OR_FAIL(c, launch_maxwell_fused(fp64, c->ndim, L, c->d_pencil + 3 * (nin + 1), c->pencil_total[3], filtered,
                                                  c->stream));
-            launches += 2;
+            launches += 1;
+            fused = true;
         } else if (ants.empty()) {
             CUDA_OR_FAIL(c, launch_maxwell(fp64, c->opt.solver, L, filtered, c->stream));
             launches += 3;
@@ -1334,7 +1338,7 @@ static pic_status enqueue_step(pic_ctx *c, int mask)
             launches += 3 + 7 * (int)ants.size();
         }
         for (int a = 0; a < 3; ++a)
-            if (c->any_periodic[a]) {
+            if (c->any_periodic[a] && !fused) {
                 CUDA_OR_FAIL(c, launch_ghost(fp64, L, a, c->ghost_max, c->stream));
                 launches++;
             }
@@ -1381,12 +1385,11 @@ extern "C" pic_status pic_step(pic_ctx *ctx, int n)
     }
     if (ctx->is_batch && ctx->persistent && !ctx->profiling && n > 0) {
         // every step in one launch of the persistent kernel
-        const int nin = (int)ctx->members.size();
         const pic_ctx *m0 = ctx->members[0];
         const int filtered = ctx->max_sweeps > 0 ? 1 : 0;
         CUDA_OR_FAIL(ctx, ctx->plan->launch(ctx->L, ctx->ndim, ctx->order, n, m0->opt.filter_passes, filtered, ctx->d_pencil,
-                                            ctx->d_pencil + 3 * (nin + 1), ctx->persist_smem, ctx->persist_grid,
-                                            ctx->spin_limit, ctx->stall_inst, ctx->stream));
+                                            ctx->persist_smem, ctx->persist_grid, ctx->spin_limit, ctx->stall_inst,
+                                            ctx->stream));
         ctx->step += n;
         ctx->mx_phases += n;
         for (auto m : ctx->members) m->step += n, m->mx_phases += n, m->last_filtered = filtered;
@@ -2144,11 +2147,15 @@ static pic_status refresh_batch(pic_ctx *c)
     if (!stale) return PIC_OK;
     const int n = (int)c->members.size();
     std::vector<InstDev> insts(n);
+    std::vector<int> cells(3 * (size_t)n);
+    for (int i = 0; i < 3 * n; ++i) cells[i] = c->members[i / 3]->n[i % 3];
+    const int planes = maxwell_planes((const int(*)[3])cells.data(), n, c->ndim, c->fp64);
     std::vector<int> ts(n + 1, 0);
     std::vector<long long> cs(n + 1, 0);
     for (int i = 0; i < n; ++i) {
         insts[i] = c->members[i]->h;
         insts[i].tile_base = ts[i];
+        insts[i].mx_planes = planes;
         ts[i + 1] = ts[i] + insts[i].ntiles;
         cs[i + 1] = cs[i] + c->members[i]->ncell;
     }
@@ -2157,7 +2164,10 @@ static pic_status refresh_batch(pic_ctx *c)
     CUDA_OR_FAIL(c, cudaMemcpyAsync(c->d_cell_start, cs.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, c->stream));
     std::vector<long long> ps((size_t)4 * (n + 1), 0);
     for (int a = 0; a < 4; ++a) {
-        for (int i = 0; i < n; ++i) ps[(size_t)a * (n + 1) + i + 1] = ps[(size_t)a * (n + 1) + i] + c->members[i]->pencil_total[a];
+        for (int i = 0; i < n; ++i)
+            ps[(size_t)a * (n + 1) + i + 1] =
+                ps[(size_t)a * (n + 1) + i] + (a < 3 ? c->members[i]->pencil_total[a]
+                                                     : maxwell_tiles(c->members[i]->n, c->ndim, planes));
         c->pencil_total[a] = ps[(size_t)a * (n + 1) + n];
     }
     CUDA_OR_FAIL(c, cudaMemcpyAsync(c->d_pencil, ps.data(), sizeof(long long) * ps.size(), cudaMemcpyHostToDevice, c->stream));
@@ -2206,10 +2216,10 @@ extern "C" pic_status pic_batch_set_persistent(pic_ctx *batch, int on, long long
                 const int o1 = a == 0 ? 1 : 0, o2 = a == 2 ? 1 : 2;
                 k.ghost[a] = m->any_periodic[a] ? 6LL * 2 * m->h.gh[a] * m->h.P[o1] * m->h.P[o2] : 0;
             }
-            k.mx_tiles = m->pencil_total[3];
+            for (int a = 0; a < 3; ++a) k.n[a] = m->n[a];
         }
         PersistPlan *plan = new PersistPlan;
-        cudaError_t e = plan->build(counts, plan_alloc, batch);
+        cudaError_t e = plan->build(batch->ndim, counts, plan_alloc, batch);
         if (e != cudaSuccess) {
             delete plan;
             return fail(batch, e == cudaErrorMemoryAllocation ? PIC_ERR_OOM : PIC_ERR_CUDA, "work list: %s", cudaGetErrorString(e));

@@ -127,6 +127,8 @@ struct InstDev {
     void *E[3], *B[3], *J[3], *Jt[3];  // Jt: scratch for filter sweeps
     void *E2[3], *B2[3];               // the second E / B buffer
     int *fpar;                         // 0: E, B current; 1: E2, B2
+    int *mx_done;                      // CTAs of the fused Maxwell update completed
+    int mx_planes;                     // its planes per z chunk (maxwell_planes)
     // particles, two buffers
     int *cell[2];
     void *off[2][3];

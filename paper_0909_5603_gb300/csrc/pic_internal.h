@@ -95,7 +95,7 @@ struct PersistCounts {
     long long ncell;
     int ntiles;
     long long pencils[3];  // filter pencils per axis
-    long long mx_tiles;    // fused Yee tiles
+    int n[3];              // cells per axis
     long long ghost[3];    // periodic ghost-copy elements per axis (0: not periodic)
 };
 // The device work list of a batch (per-phase item offsets and the launch's counters).
@@ -107,14 +107,13 @@ class PersistPlan {
     PersistPlan(const PersistPlan &) = delete;
     PersistPlan &operator=(const PersistPlan &) = delete;
     // device memory from alloc(user, bytes), owned by the caller's context
-    cudaError_t build(const std::vector<PersistCounts> &inst, void *(*alloc)(void *, size_t), void *user);
+    cudaError_t build(int ndim, const std::vector<PersistCounts> &inst, void *(*alloc)(void *, size_t), void *user);
     long long items_per_step() const;
     // nsteps steps of the batch in one launch of grid CTAs (kNT threads, smem bytes of
-    // dynamic shared memory); pencil_tables: the three per-axis pencil offset tables,
-    // mx_start: the fused Yee tile offsets
+    // dynamic shared memory); pencil_tables: the three per-axis pencil offset tables
     cudaError_t launch(const Launch &L, int ndim, int order, int nsteps, int passes, int filtered,
-                       const long long *pencil_tables, const long long *mx_start, size_t smem, int grid,
-                       long long spin_limit, int stall_inst, cudaStream_t s);
+                       const long long *pencil_tables, size_t smem, int grid, long long spin_limit, int stall_inst,
+                       cudaStream_t s);
 
   private:
     Impl *impl;
@@ -125,15 +124,58 @@ cudaError_t persist_blocks_per_sm(int ndim, int order, size_t smem, int *bps);
 
 // opt-in to the shared memory of the fused Yee update (once per device and precision)
 cudaError_t prepare_fields(int fp64);
-// the whole Yee update of the step (Yee solver, no antenna) in one launch over
-// maxwell_tiles() tiles per instance, then the switch of every instance to the E / B
-// buffer pair it wrote
+// Columns of a block of the fused Yee update, and the blocks of an SM: 32 x 8 columns in
+// 3D; in 2D3V 64, so that a narrow grid fills its blocks and several small blocks hide one
+// another's barriers (128 x 128 cells, FP32: 46 us with one block of 256 columns per 32
+// planes).
+template <int ND>
+struct MxTile;
+template <>
+struct MxTile<3> {
+    static constexpr int X = 32, Y = 8;
+};
+template <>
+struct MxTile<2> {
+    static constexpr int X = 64, Y = 1;
+};
+template <typename R, int ND>
+constexpr int mx_resident()
+{
+    return ND == 3 ? (sizeof(R) == 4 ? 3 : 2) : (sizeof(R) == 4 ? 12 : 7);
+}
+// the whole Yee update of the step (Yee solver, no antenna) with its periodic images in one
+// launch over maxwell_tiles() tiles per instance; each instance ends on the E / B buffer
+// pair it wrote
 cudaError_t launch_maxwell_fused(int fp64, int ndim, const Launch &L, const long long *tile_start, long long ntiles,
                                  int filtered, cudaStream_t s);
-inline long long maxwell_tiles(const int n[3], int ndim)
+inline long long maxwell_tiles(const int n[3], int x, int y, int planes)
 {
-    return ndim == 3 ? (long long)((n[0] + 31) / 32) * ((n[1] + 7) / 8) * ((n[2] + 31) / 32)
-                     : (long long)((n[0] + 255) / 256) * ((n[2] + 31) / 32);
+    return (long long)((n[0] + x - 1) / x) * ((n[1] + y - 1) / y) * ((n[2] + planes - 1) / planes);
+}
+inline long long maxwell_tiles(const int n[3], int ndim, int planes)
+{
+    return ndim == 3 ? maxwell_tiles(n, MxTile<3>::X, MxTile<3>::Y, planes) : maxwell_tiles(n, MxTile<2>::X, MxTile<2>::Y, planes);
+}
+// Planes per z chunk for a launch over `count` instances of n[i] cells.  A block works
+// through its planes one after the other behind a prologue of about four, so the launch
+// takes about waves x (planes + 4) plane times (1 to 4 us each): long chunks leave a small
+// grid on a few SMs, short ones repeat the prologue.
+inline int maxwell_planes(const int (*n)[3], int count, int ndim, int fp64)
+{
+    const long long slots = 152LL * (ndim == 3 ? (fp64 ? mx_resident<double, 3>() : mx_resident<float, 3>())
+                                               : (fp64 ? mx_resident<double, 2>() : mx_resident<float, 2>()));
+    int best = 2;
+    long long least = -1;
+    for (int p = 2; p <= 64; ++p) {
+        long long tiles = 0;
+        for (int i = 0; i < count; ++i) tiles += maxwell_tiles(n[i], ndim, p);
+        const long long cost = (tiles + slots - 1) / slots * (p + 4);
+        if (least < 0 || cost <= least) {
+            least = cost;
+            best = p;
+        }
+    }
+    return best;
 }
 // passes: the filter passes of every instance of the launch (0 when they differ)
 cudaError_t launch_filter(int fp64, const Launch &L, const long long *const pencil_start[3],
