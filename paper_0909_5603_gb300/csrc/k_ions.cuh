@@ -63,16 +63,19 @@ __device__ __forceinline__ void ion_faces_of(const InstDev &I, int first, int st
     }
 }
 
-// Jz of interior cell r (x fastest) of instance I <- the ion current of its plane.
+// J of interior cell r (x fastest) of instance I at the start of a step: zero, and on Jz
+// the ion current of its plane.
 template <typename R>
-__device__ __forceinline__ void ion_current_cell(const InstDev &I, int r)
+__device__ __forceinline__ void j_init_cell(const InstDev &I, int r)
 {
     const int rq = fast_div(r, I.div_n0);
     const int i = r - rq * I.n[0];
     const int k = fast_div(rq, I.div_n1);
     const int j = rq - k * I.n[1];
     const long long p = (i + I.gh[0]) + I.sy * (j + I.gh[1]) + I.sz * (k + I.gh[2]);
-    ((R *)I.J[2])[p] = ((const R *)I.ion_face)[k];
+    ((R *)I.J[0])[p] = R(0);
+    ((R *)I.J[1])[p] = R(0);
+    ((R *)I.J[2])[p] = I.ion ? ((const R *)I.ion_face)[k] : R(0);
 }
 
 }  // namespace pic

@@ -177,16 +177,8 @@ __global__ void __launch_bounds__(kNT, 2) k_step_persistent(Launch L, PersistDes
             break;
         case kPhJInit: {
             const long long ncell = (long long)I.n[0] * I.n[1] * I.n[2];
-            for (long long r = local * kJInitCells + tid; r < min(ncell, (local + 1) * kJInitCells); r += kNT) {
-                const int rq = fast_div((int)r, I.div_n0);
-                const int i = (int)r - rq * I.n[0];
-                const int k = fast_div(rq, I.div_n1);
-                const int j = rq - k * I.n[1];
-                const long long pc = (i + I.gh[0]) + I.sy * (j + I.gh[1]) + I.sz * (k + I.gh[2]);
-                ((float *)I.J[0])[pc] = 0.f;
-                ((float *)I.J[1])[pc] = 0.f;
-                ((float *)I.J[2])[pc] = I.ion ? ((const float *)I.ion_face)[k] : 0.f;
-            }
+            for (long long r = local * kJInitCells + tid; r < min(ncell, (local + 1) * kJInitCells); r += kNT)
+                j_init_cell<float>(I, (int)r);
             break;
         }
         case kPhScan:
