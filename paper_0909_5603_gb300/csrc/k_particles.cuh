@@ -1109,6 +1109,16 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
     if (PARTS && split >= 0) close_parts(I, out, t, split, count, pch, chunk_out, S);
 }
 
+// Blocks per SM that the registers of the particle kernel are bounded for.  The 2D3V body
+// fits 80 registers with 12 bytes of spills (a launch of one instance), so three blocks of
+// 256 threads hide more of one another's waits (a batch of 32 instances: 1.21 -> 1.15 ms); the
+// 3D one would spill 230 bytes, which costs more than the warps give (4.45 against 4.19 ms).
+template <int ND, typename R>
+constexpr int particle_blocks()
+{
+    return sizeof(R) == 4 ? (ND == 2 ? 3 : 2) : 1;
+}
+
 // the particle phase of tile g of the launch (its global index over the instances)
 template <int ND, int ORD, typename R, int PUSHER, bool INJ>
 __device__ __forceinline__ void particle_tile_of_launch(const Launch &L, const int g)
@@ -1118,9 +1128,18 @@ __device__ __forceinline__ void particle_tile_of_launch(const Launch &L, const i
 }
 
 template <int ND, int ORD, typename R, int PUSHER, bool INJ>
-__global__ void __launch_bounds__(kNT, sizeof(R) == 4 ? 2 : 1) k_particles(Launch L)
+__global__ void __launch_bounds__(kNT, particle_blocks<ND, R>()) k_particles(Launch L)
 {
-    particle_tile_of_launch<ND, ORD, R, PUSHER, INJ>(L, blockIdx.x);
+    // the instance in shared memory: from the device array its fields were loaded again after
+    // every particle store, which may alias them (a batch of 32 instances: 1.31 -> 1.21 ms)
+    __shared__ InstDev I;
+    const int g = blockIdx.x;
+    const int ii = find_instance(L.tile_start, L.ninst, g);
+    static_assert(sizeof(InstDev) % 8 == 0, "copied in 8-byte words");
+    const uint64_t *src = reinterpret_cast<const uint64_t *>(L.inst + ii);
+    for (int e = threadIdx.x; e < (int)(sizeof(InstDev) / 8); e += kNT) reinterpret_cast<uint64_t *>(&I)[e] = src[e];
+    __syncthreads();
+    particle_tile<ND, ORD, R, PUSHER, INJ, false, false>(I, g - L.tile_start[ii], 0);
 }
 
 // a launch of one instance: the instance by value.  The first I.over_max blocks take the
@@ -1128,7 +1147,7 @@ __global__ void __launch_bounds__(kNT, sizeof(R) == 4 ? 2 : 1) k_particles(Launc
 // others one tile each.  (A bunch of 2^20 electrons in 64x64x256 cells, 133,000 of them in
 // one tile: 0.19 ms instead of the 1.14 ms that one CTA needs for that tile.)
 template <int ND, int ORD, typename R, int PUSHER, bool INJ>
-__global__ void __launch_bounds__(kNT, sizeof(R) == 4 ? 2 : 1) k_particles_one(const __grid_constant__ InstDev I)
+__global__ void __launch_bounds__(kNT, particle_blocks<ND, R>()) k_particles_one(const __grid_constant__ InstDev I)
 {
     int t = (int)blockIdx.x - I.over_max, part = 0;
     if (t < 0) {
