@@ -116,17 +116,6 @@ __device__ __forceinline__ int axis_sources(int T, int nt, int bc, int dirs[3], 
     return m;
 }
 
-// Canonical direction along one axis from old tile coordinate to new one.
-__device__ __forceinline__ int axis_dir(int told, int tnew, int nt, int bc)
-{
-    if (bc != 0) return tnew - told;
-    int d = tnew - told;
-    if (d < 0) d += nt;  // d in [0, nt)
-    if (d == 0) return 0;
-    if (d == 1) return 1;
-    return -1;           // d == nt - 1 with nt >= 3
-}
-
 // The last chunk k of [0, nch) whose count of bucket d in the tile's earlier chunks (cb,
 // the tile's first record) is at most j: the chunk that holds the tile's j-th particle of
 // that bucket.
@@ -273,6 +262,27 @@ __device__ __forceinline__ int slot_position(const InstDev &I, int lay, const Sr
     const int lo = chunk_of(cb + (long long)S.c0[s] * kBuckets, S.nch[s], d, j);
     const long long c = S.c0[s] + lo;
     return S.seg[s] + lo * I.R + I.chunk_pre[lay][c * kPre + d] + (j - cb[c * kBuckets + d]);
+}
+
+// Buffer position of slot p (-1 without a particle) for the lanes of a warp at consecutive
+// slots from p0 on.  With at most 64 sub-ranges the one of p0 is found by the warp together
+// (two votes) and each lane walks on from there, a step or two: sub-ranges are tens of
+// slots long.  Called by the whole warp.
+__device__ __forceinline__ int slot_position_warp(const InstDev &I, int lay, const SrcTable &S, int p0, int p, bool live,
+                                                  int lane)
+{
+    if ((unsigned)S.nsub > 64u) return live ? slot_position(I, lay, S, p) : -1;
+    const int n = S.nsub;
+    const unsigned v0 = __ballot_sync(0xffffffffu, lane < n && S.sub_slot[lane] <= p0);
+    const unsigned v1 = __ballot_sync(0xffffffffu, lane + 32 < n && S.sub_slot[lane + 32] <= p0);
+    if (!live) return -1;
+    int e = __popc(v0) + __popc(v1) - 1;
+    int at = S.sub_slot[e];
+    for (int next = S.sub_slot[e + 1]; next <= p; next = S.sub_slot[e + 1]) {  // (ends at sub_slot[n] > p)
+        ++e;
+        at = next;
+    }
+    return S.sub_pos[e] + (p - at);
 }
 
 // -------------------------------------------------------------------------------------
@@ -674,10 +684,18 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
     __shared__ uint64_t bar;
     __shared__ int s_run[kBuckets];          // running bucket totals of the tile (warp 0)
     // each thread's particle of the next chunk, copied in (cp.async) while the current
-    // chunk is processed; two buffers, chunk r in buffer r & 1
-    __shared__ int s_pcell[2][kNT], s_pid[2][kNT];
-    __shared__ R s_poff[2][3][kNT], s_pu[2][3][kNT], s_pw[2][kNT];
-    __shared__ int s_cnt[2][kNW][kBuckets];  // per-warp bucket counts, double-buffered per chunk
+    // chunk is processed.  A thread reads its own entries only and takes them into registers
+    // before it stages the next ones, so one buffer does (128x128x1024 stage: 4.19 ms, with
+    // two 4.27); where entries are read again during the chunk (spread lanes, frozen beam
+    // particles) there are two, chunk r in buffer r & 1
+    constexpr bool kSpread = kFixed && ND == 2;
+    constexpr int NB = kSpread || INJ ? 2 : 1;
+    __shared__ int s_pcell[NB][kNT], s_pid[NB][kNT];
+    __shared__ R s_poff[NB][3][kNT], s_pu[NB][3][kNT], s_pw[NB][kNT];
+    // per-warp bucket counts, one byte each (at most 32), double-buffered per chunk: the eight
+    // warps' counts of a bucket are one 8-byte word
+    static_assert(kNW == 8, "a bucket's counts are one word");
+    __shared__ __align__(8) unsigned char s_cnt[2][32][kNW];
     __shared__ __align__(16) unsigned s_bmax[3][kNW];  // FP32: per-warp contribution bounds of the chunk
 
     const int out = *I.cur;  // the scan of this step already flipped the parity
@@ -739,7 +757,6 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
     }
     for (int e = tid; e < 2 * jv4; e += kNT)  // A and T (or the FP64 tile)
         reinterpret_cast<int4 *>(sJraw)[e] = make_int4(0, 0, 0, 0);
-    for (int e = tid; e < 2 * kNW * kBuckets; e += kNT) (&s_cnt[0][0][0])[e] = 0;
     if (tid < kBuckets) s_run[tid] = 0;
     // the tile's source table: its precomputed record (one coalesced read), or built here
     // when the record overflowed
@@ -768,78 +785,103 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
     // per-instance constants in the working precision (host-formed); in FP32 mode the
     // current factor qdv carries the fixed-point scale (see ChunkAcc)
     const StepCoef<R> &K = coef<R>(I);
-    const R h = K.h;
-    const R qdv = K.qdv;
-    const R jfx = K.jf[0], jfy = K.jf[1], jfz = K.jf[2];
-    const R dtdx[3] = {K.dtdx[0], K.dtdx[1], K.dtdx[2]};
     // beam injection plane in cells along z at this step's push time t^n = n dt (n: the
     // phases before this one), in FP64; beam particles upstream of it are frozen
     const bool inj = INJ && I.inj_id0 != INT_MAX;
     double zp_inj = 0.0;
     if (inj) zp_inj = (I.inj_zb - I.beta_b * ((double)(*I.phase - 1) * I.dt)) / I.dx[2];
-    const int bx = I.box[0], bxy = I.box[0] * I.box[1];
-    const int jd0 = I.jdim[0], jd01 = I.jdim[0] * I.jdim[1];
-    const int jlo_y = ND == 3 ? I.jlo : 0;
     const int tsx = min(I.ts[0], I.n[0] - T0[0]);
     const int tsy = min(I.ts[1], I.n[1] - T0[1]);
     const int tsz = min(I.ts[2], I.n[2] - T0[2]);
 
-    const int *cell_in = I.cell[in];
-    const R *off_in[3] = {(const R *)I.off[in][0], (const R *)I.off[in][1], (const R *)I.off[in][2]};
-    const R *u_in[3] = {(const R *)I.u[in][0], (const R *)I.u[in][1], (const R *)I.u[in][2]};
-    const R *w_in = (const R *)I.w[in];
-    const int *id_in = I.id[in];
-    int *cell_out = I.cell[out];
-    R *off_out[3] = {(R *)I.off[out][0], (R *)I.off[out][1], (R *)I.off[out][2]};
-    R *u_out[3] = {(R *)I.u[out][0], (R *)I.u[out][1], (R *)I.u[out][2]};
-    R *w_out = (R *)I.w[out];
-    int *id_out = I.id[out];
+    // the bucket's change when a particle leaves the tile below or above along an axis (the
+    // canonical direction: with two periodic tiles both ways are +1, with one it stays), and
+    // whether the tile touches a face of the box
+    int dir_lo[3], dir_hi[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int st = a == 0 ? 1 : a == 1 ? 3 : 9;
+        const bool apart = I.bc[a] != 0 || I.nt[a] >= 3;
+        dir_lo[a] = apart ? -st : I.nt[a] == 2 ? st : 0;
+        dir_hi[a] = apart || I.nt[a] == 2 ? st : 0;
+    }
+    const bool at_face = tx == 0 || tx == I.nt[0] - 1 || tz == 0 || tz == I.nt[2] - 1 ||
+                         (ND == 3 && (ty == 0 || ty == I.nt[1] - 1));
+
+    // (what the loop needs of I is read where it is used: the particle arrays' addresses alone
+    // would take 40 registers across the loop)
+    const bool ids = I.id[in] != nullptr;
 
     // stages this thread's particle of slot first + sl into buffer b of the s_p* arrays
     // (asynchronously); returns its position in the input buffer, or -1
     auto stage = [&](int sl, int b) -> int {
-        const int p = sl < mine ? slot_position(I, in, S, first + sl) : -1;
+        const int p = slot_position_warp(I, in, S, first + sl - lane, first + sl, sl < mine, lane);
         if (p >= 0 && p < I.cap) {
-            cp_async<4>(&s_pcell[b][tid], cell_in + p);
-            cp_async<sizeof(R)>(&s_poff[b][0][tid], off_in[0] + p);
-            if (ND == 3) cp_async<sizeof(R)>(&s_poff[b][1][tid], off_in[1] + p);
-            cp_async<sizeof(R)>(&s_poff[b][2][tid], off_in[2] + p);
-            cp_async<sizeof(R)>(&s_pu[b][0][tid], u_in[0] + p);
-            cp_async<sizeof(R)>(&s_pu[b][1][tid], u_in[1] + p);
-            cp_async<sizeof(R)>(&s_pu[b][2][tid], u_in[2] + p);
-            cp_async<sizeof(R)>(&s_pw[b][tid], w_in + p);
-            if (id_in) cp_async<4>(&s_pid[b][tid], id_in + p);
+            cp_async<4>(&s_pcell[b][tid], I.cell[in] + p);
+            cp_async<sizeof(R)>(&s_poff[b][0][tid], (const R *)I.off[in][0] + p);
+            if (ND == 3) cp_async<sizeof(R)>(&s_poff[b][1][tid], (const R *)I.off[in][1] + p);
+            cp_async<sizeof(R)>(&s_poff[b][2][tid], (const R *)I.off[in][2] + p);
+            cp_async<sizeof(R)>(&s_pu[b][0][tid], (const R *)I.u[in][0] + p);
+            cp_async<sizeof(R)>(&s_pu[b][1][tid], (const R *)I.u[in][1] + p);
+            cp_async<sizeof(R)>(&s_pu[b][2][tid], (const R *)I.u[in][2] + p);
+            cp_async<sizeof(R)>(&s_pw[b][tid], (const R *)I.w[in] + p);
+            if (ids) cp_async<4>(&s_pid[b][tid], I.id[in] + p);
         }
         cp_async_commit();
         return p;
     };
     int pos_next = stage(tid, 0);
     float inv[3] = {1.f, 1.f, 1.f};  // FP32: the current chunk's per-component 1 / scale
+    // FP32, 2D3V: the deposit's lanes.  The particles of a tile are nearly sorted by cell, so
+    // with many particles per cell the lanes of a warp share a few window starts, and shared
+    // atomics serialise lanes on one address (a bank model on sorted particles gives, per
+    // add, 6.7 wavefronts with 9 and 9.7 with 16 particles per cell, 3.4 and 3.6 for spread
+    // ones).  From 4 particles per cell on (model: 4.3 and 3.2), thread tid therefore deposits
+    // the particle of slot dslot of the chunk, handed over through its staging buffer: a
+    // warp's lanes take slots about 8 apart over the whole chunk, on 32 different banks.  The
+    // gather keeps the sorted lanes, which read the same field values.  A batch of 32
+    // instances with 1 to 16 particles per cell: 1.05 instead of 1.14 ms.  (In 3D the same
+    // hand-over gained nothing with 16 particles per cell, 674 against 663 us.)
+    const bool spread = kSpread && count >= 4 * tsx * tsy * tsz;
+    const int dslot = 32 * (lane >> 2) + 8 * (lane & 3) + (((lane >> 2) + warp) & 7);
 
     for (int base = 0, r = 0; base < mine; base += kChunk, ++r) {
+        const R h = K.h;
+        const R qdv = K.qdv;
+        const R jfx = K.jf[0], jfy = K.jf[1], jfz = K.jf[2];
+        const R dtdx[3] = {K.dtdx[0], K.dtdx[1], K.dtdx[2]};
+        const int bx = I.box[0], bxy = I.box[0] * I.box[1];
+        const int jd0 = I.jdim[0], jd01 = I.jdim[0] * I.jdim[1];
+        const int jlo_y = ND == 3 ? I.jlo : 0;
         int bucket = 28;  // 0..26 direction, 27 dead, 28 no particle
         int cell_new = 0, pid = 0;
         R o1[3] = {R(0), R(0), R(0)}, u[3] = {R(0), R(0), R(0)}, w = R(0);
         const int slot = base + tid;
         const int pos = pos_next;
-        const int pb = r & 1;
+        const int pb = r & (NB - 1);
         cp_async_wait_all();  // this thread's particle of this chunk has landed
-        if (base + kChunk < mine) pos_next = stage(base + kChunk + tid, pb ^ 1);
+        const int cell = s_pcell[pb][tid], pid_in = ids ? s_pid[pb][tid] : 0;
+        const R po[3] = {s_poff[pb][0][tid], ND == 3 ? s_poff[pb][1][tid] : R(0), s_poff[pb][2][tid]};
+        const R pu[3] = {s_pu[pb][0][tid], s_pu[pb][1][tid], s_pu[pb][2][tid]};
+        const R pw = s_pw[pb][tid];
+        if (base + kChunk < mine) pos_next = stage(base + kChunk + tid, (r + 1) & (NB - 1));
         if (slot < mine && (pos < 0 || pos >= I.cap)) atomicOr(I.err, kErrInternal);
         int l[3] = {0, 0, 0}, cc[3] = {0, 0, 0};
         // deposit inputs
         R o[3] = {R(0.5), R(0.5), R(0.5)};
         int l1[3] = {0, 0, 0};
         R disp[3] = {R(0), R(0), R(0)};
-        R fx = R(0), fy = R(0), fz = R(0);
+        R fx = R(0), fy = R(0), fz = R(0), vy = R(0);
+        int db[3] = {0, 0, 0};
         o1[0] = o1[1] = o1[2] = R(0.5);
         bool have = false;
         if (pos >= 0 && pos < I.cap) {
-            const int c = s_pcell[pb][tid];
+            const int c = cell;
             const int cyz = fast_div(c, I.div_n0);
             cc[0] = c - cyz * I.n[0];
-            cc[2] = fast_div(cyz, I.div_n1);
-            cc[1] = cyz - cc[2] * I.n[1];
+            cc[2] = ND == 3 ? fast_div(cyz, I.div_n1) : cyz;
+            cc[1] = ND == 3 ? cyz - cc[2] * I.n[1] : 0;
+            cell_new = c;
             l[0] = cc[0] - T0[0];
             l[1] = cc[1] - T0[1];
             l[2] = cc[2] - T0[2];
@@ -847,14 +889,10 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
             if (!have) atomicOr(I.err, kErrInternal);
         }
         if (have) {
-            o[0] = s_poff[pb][0][tid];
-            o[1] = ND == 3 ? s_poff[pb][1][tid] : R(0);
-            o[2] = s_poff[pb][2][tid];
-            u[0] = s_pu[pb][0][tid];
-            u[1] = s_pu[pb][1][tid];
-            u[2] = s_pu[pb][2][tid];
-            w = s_pw[pb][tid];
-            pid = id_in ? s_pid[pb][tid] : 0;
+            o[0] = po[0], o[1] = po[1], o[2] = po[2];
+            u[0] = pu[0], u[1] = pu[1], u[2] = pu[2];
+            w = pw;
+            pid = pid_in;
 
             // ---- gather (Yee positions: E_a staggered along a, B_a along the other two)
             R E[3], B[3];
@@ -902,7 +940,6 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
             bool bad = false;
             o1[0] = o[0]; o1[1] = o[1]; o1[2] = o[2];
             int kstep[3] = {0, 0, 0};
-            R vy;
             if (sizeof(R) == 4) {
                 const float gn = sqrtf(1.f + (float)u[0] * (float)u[0] + (float)u[1] * (float)u[1] + (float)u[2] * (float)u[2]);
                 const float ig = 1.f / gn;
@@ -935,43 +972,39 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
                 l1[0] = l[0] + kstep[0];
                 l1[1] = l[1] + kstep[1];
                 l1[2] = l[2] + kstep[2];
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    db[a] = kstep[a] + (ORD == 2 ? (o1[a] >= R(0.5) ? 1 : 0) - (o[a] >= R(0.5) ? 1 : 0) : 0);
                 const R qw = qdv * w;
                 fx = -qw * jfx;
                 fy = ND == 3 ? -qw * jfy : qw * vy;
                 fz = -qw * jfz;
             }
 
-            // ---- new cell, destination tile, bucket
-            int cn[3] = {cc[0] + kstep[0], cc[1] + kstep[1], cc[2] + kstep[2]};
-            bool dead = false;
+            // ---- new cell and bucket, the direction of the new tile: a move stays below one
+            // cell, so that is this tile or, below or above its cells, a neighbour
+            cell_new += kstep[0] + I.n[0] * (kstep[1] + I.n[1] * kstep[2]);
+            bucket = kCenterDir;
+            const int tl[3] = {tsx, tsy, tsz};
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 if (ND == 2 && a == 1) continue;
-                if (cn[a] < 0 || cn[a] >= I.n[a]) {
-                    if (I.bc[a] == 0)
-                        cn[a] += cn[a] < 0 ? I.n[a] : -I.n[a];
-                    else
-                        dead = true;
-                }
+                bucket += l1[a] < 0 ? dir_lo[a] : (l1[a] >= tl[a] ? dir_hi[a] : 0);
             }
-            if (dead) {
-                bucket = kDead;
-            } else {
-                // the new tile from the tile-local cell (a move stays below one cell, so it
-                // is this tile or a neighbour; across a periodic face the coordinate wraps)
-                const int l1v[3] = {l[0] + kstep[0], l[1] + kstep[1], l[2] + kstep[2]};
-                const int tl[3] = {tsx, tsy, tsz}, to[3] = {tx, ty, tz};
-                int dd[3] = {0, 0, 0};
+            if (at_face) {  // beyond a face of the box: the cell wraps, or the particle is removed
+                bool dead = false;
+                const int st[3] = {1, I.n[0], I.n[0] * I.n[1]};
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     if (ND == 2 && a == 1) continue;
-                    int tn = to[a] + (l1v[a] < 0 ? -1 : (l1v[a] >= tl[a] ? 1 : 0));
-                    tn += tn < 0 ? I.nt[a] : (tn >= I.nt[a] ? -I.nt[a] : 0);
-                    dd[a] = axis_dir(to[a], tn, I.nt[a], I.bc[a]);
+                    const int cn = cc[a] + kstep[a];
+                    if (cn < 0 || cn >= I.n[a]) {
+                        cell_new += (cn < 0 ? I.n[a] : -I.n[a]) * st[a];
+                        dead = dead || I.bc[a] != 0;
+                    }
                 }
-                bucket = (dd[2] + 1) * 9 + (dd[1] + 1) * 3 + (dd[0] + 1);
+                if (dead) bucket = kDead;
             }
-            cell_new = cn[0] + I.n[0] * (cn[1] + I.n[1] * cn[2]);
         }
 
         // ---- Esirkepov deposit into the shared J tile, by the lanes that hold a particle: in
@@ -994,59 +1027,88 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
                 const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(bnd[a]));
                 if (lane == 0) s_bmax[a][warp] = m;
             }
+            if (spread) {
+                // the offsets and the weight are still in the staging buffer
+                s_pcell[pb][tid] = !have ? 0
+                                         : 1 << 24 | l[0] | l[1] << 6 | l[2] << 12 | (db[0] + 1) << 18 | (db[1] + 1) << 20 |
+                                               (db[2] + 1) << 22;
+                s_pu[pb][0][tid] = disp[0];
+                s_pu[pb][1][tid] = ND == 3 ? disp[1] : vy;
+                s_pu[pb][2][tid] = disp[2];
+            }
             __syncthreads();
+            // lanes 8 a .. 8 a + 7 form component a's scale from the warps' bounds
             float sc[3];
+            {
+                unsigned m = (&s_bmax[0][0])[lane < 3 * kNW ? lane : 0];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const uint4 m0 = reinterpret_cast<const uint4 *>(s_bmax[a])[0];
-                const uint4 m1 = reinterpret_cast<const uint4 *>(s_bmax[a])[1];
-                const unsigned m = max(max(max(m0.x, m0.y), max(m0.z, m0.w)), max(max(m1.x, m1.y), max(m1.z, m1.w)));
+                for (int o = 1; o < kNW; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
                 // the largest contribution is at most K times the bound (see ChunkAcc): K =
                 // S_max^2 in 3D and for the out-of-plane current of 2D3V, S_max for the
                 // in-plane ones; S_max = 3/4 (order 2) or 1 (order 1)
                 constexpr float Smax = ORD == 2 ? 0.75f : 1.0f;
-                const float K = (ND == 3 || a == 1) ? Smax * Smax : Smax;
+                const float K = (ND == 3 || lane / kNW == 1) ? Smax * Smax : Smax;
                 // inv = K bound / (0.999 2^22), scale = 1 / inv (correctly rounded, so
                 // scale x inv = 1 to FP32 precision)
                 const float bk = K * __uint_as_float(m);
-                inv[a] = bk > 1e-30f ? bk * (1.0f / (0.999f * 4194304.0f)) : 1.0f;
-                sc[a] = __frcp_rn(inv[a]);
+                const float iv = bk > 1e-30f ? bk * (1.0f / (0.999f * 4194304.0f)) : 1.0f;
+                const float s = __frcp_rn(iv);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    inv[a] = __shfl_sync(0xffffffffu, iv, kNW * a);
+                    sc[a] = __shfl_sync(0xffffffffu, s, kNW * a);
+                }
             }
             // the current follows the computed displacement (see shape_window)
-            const unsigned lanes = __ballot_sync(0xffffffffu, have);
-            if (have)
-                deposit_esirkepov<ND, ORD, true, true, LANEWIN, R>(lanes, l, o, l1, o1, disp, fx * sc[0], fy * sc[1],
+            bool dep = have;
+            if (spread) {
+                const int c = s_pcell[pb][dslot];
+                dep = c != 0;
+                l[0] = c & 63, l[1] = (c >> 6) & 63, l[2] = (c >> 12) & 63;
+                db[0] = ((c >> 18) & 3) - 1, db[1] = ((c >> 20) & 3) - 1, db[2] = ((c >> 22) & 3) - 1;
+                o[0] = s_poff[pb][0][dslot];
+                o[1] = ND == 3 ? s_poff[pb][1][dslot] : R(0);
+                o[2] = s_poff[pb][2][dslot];
+                disp[0] = s_pu[pb][0][dslot];
+                disp[1] = ND == 3 ? s_pu[pb][1][dslot] : R(0);
+                disp[2] = s_pu[pb][2][dslot];
+                const R qw = qdv * s_pw[pb][dslot];
+                fx = -qw * jfx;
+                fy = ND == 3 ? -qw * jfy : qw * s_pu[pb][1][dslot];
+                fz = -qw * jfz;
+            }
+            const unsigned lanes = __ballot_sync(0xffffffffu, dep);
+            if (dep)
+                deposit_esirkepov<ND, ORD, true, true, LANEWIN, R>(lanes, l, o, l1, o1, db, disp, fx * sc[0], fy * sc[1],
                                                                    fz * sc[2], I.jlo, jlo_y, jd0, jd01, jst,
                                                                    ChunkAcc{sJA});
         } else {
             if (have)
-                deposit_esirkepov<ND, ORD, false, false, false, R>(0u, l, o, l1, o1, disp, fx, fy, fz, I.jlo, jlo_y, jd0,
+                deposit_esirkepov<ND, ORD, false, false, false, R>(0u, l, o, l1, o1, db, disp, fx, fy, fz, I.jlo, jlo_y, jd0,
                                                                    jd01, jst, DoubleAcc{sJD});
         }
 
         // ---- stable ranking of the chunk by bucket: order (warp, lane), one barrier per
-        // chunk.  Each warp writes its bucket counts into its own row of s_cnt[cbuf]
-        // (cleared by that warp first: the row was last read in chunk r - 2, before the
+        // chunk.  Each warp writes its bucket counts into its own bytes of s_cnt[cbuf]
+        // (cleared by that warp first: they were last read in chunk r - 2, before the
         // barrier of chunk r - 1), and after the barrier every warp forms the offsets it
-        // needs itself: lane d sums bucket d over the warps (its own prefix and the total),
-        // and a scan over the lanes gives the bucket bases.  Warp 0 keeps the running
-        // bucket totals of the tile and writes the chunk's records.
+        // needs itself: lane d sums the bytes of bucket d over the warps (those before its
+        // own, and all), and a scan over the lanes gives the bucket bases.  Warp 0 keeps the
+        // running bucket totals of the tile and writes the chunk's records.
         const int cbuf = r & 1;
-        if (lane < kBuckets) s_cnt[cbuf][warp][lane] = 0;
+        s_cnt[cbuf][lane][warp] = 0;
         __syncwarp();
         const unsigned peers = __match_any_sync(0xffffffffu, bucket);
         const int rank = __popc(peers & ((1u << lane) - 1u));
-        if (bucket < kBuckets && lane == __ffs(peers) - 1) s_cnt[cbuf][warp][bucket] = __popc(peers);
+        if (bucket < kBuckets && lane == __ffs(peers) - 1) s_cnt[cbuf][bucket][warp] = (unsigned char)__popc(peers);
         __syncthreads();
-        int totd = 0, below = 0;  // lane d: bucket d over all warps, and over the warps before this one
-        if (lane < kBuckets) {
-#pragma unroll
-            for (int ww = 0; ww < kNW; ++ww) {
-                const int v = s_cnt[cbuf][ww][lane];
-                below += ww < warp ? v : 0;
-                totd += v;
-            }
-        }
+        const uint2 cw = *reinterpret_cast<const uint2 *>(s_cnt[cbuf][lane]);
+        // the bytes of the warps before this one
+        const unsigned blo = warp < 4 ? (1u << (8 * warp)) - 1u : 0xffffffffu;
+        const unsigned bhi = warp < 4 ? 0u : (1u << (8 * (warp - 4))) - 1u;
+        // lane d: bucket d over all warps, and over the warps before this one
+        const int totd = (int)__dp4a(cw.x, 0x01010101u, __dp4a(cw.y, 0x01010101u, 0u));
+        const int below = (int)__dp4a(cw.x & blo, 0x01010101u, __dp4a(cw.y & bhi, 0x01010101u, 0u));
         int incl = totd;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -1068,15 +1130,15 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
         // ---- write the particle out, partitioned by bucket
         if (bucket < kDead) {
             const int p = seg_mine + base + myoff + rank;
-            cell_out[p] = cell_new;
-            off_out[0][p] = o1[0];
-            if (ND == 3) off_out[1][p] = o1[1];
-            off_out[2][p] = o1[2];
-            u_out[0][p] = u[0];
-            u_out[1][p] = u[1];
-            u_out[2][p] = u[2];
-            w_out[p] = w;
-            if (id_out) id_out[p] = pid;
+            I.cell[out][p] = cell_new;
+            ((R *)I.off[out][0])[p] = o1[0];
+            if (ND == 3) ((R *)I.off[out][1])[p] = o1[1];
+            ((R *)I.off[out][2])[p] = o1[2];
+            ((R *)I.u[out][0])[p] = u[0];
+            ((R *)I.u[out][1])[p] = u[1];
+            ((R *)I.u[out][2])[p] = u[2];
+            ((R *)I.w[out])[p] = w;
+            if (ids) I.id[out][p] = pid;
         }
 
         // ---- FP32: fold the chunk accumulator into the FP32 tile (the last chunk's is

@@ -65,15 +65,16 @@ __device__ __forceinline__ int shape_stag(int l, R o, R w[ORD + 1])
 // 3e-8 / d, 6e-6 for a thermal particle moving 0.005 cells per step.  Taking the computed
 // displacement keeps J at FP32 precision relative to the motion; the rounding then
 // appears only as a charge-conservation residual of at most half an ulp times the shape
-// slope per particle and step.  With kDisp a particle that changes its nodes gets DS from
+// slope per particle and step.  The new position (l1, o1) then enters only through db, the
+// change of the first node.  With kDisp a particle that changes its nodes gets DS from
 // the slopes over the two parts of its move (below), not from a difference of weights.
 template <int ORD, bool kDisp, typename R>
-__device__ __forceinline__ int shape_window(int l0, R o0, int l1, R o1, R disp, R S0[ORD + 2], R DS[ORD + 2],
+__device__ __forceinline__ int shape_window(int l0, R o0, int l1, R o1, int db, R disp, R S0[ORD + 2], R DS[ORD + 2],
                                             int &nw)
 {
-    R w0[ORD + 1], w1[ORD + 1];
+    R w0[ORD + 1], w1[ORD + 1] = {};
     const int b0 = shape_nodal<ORD>(l0, o0, w0);
-    const int b1 = shape_nodal<ORD>(l1, o1, w1);
+    const int b1 = kDisp ? b0 + db : shape_nodal<ORD>(l1, o1, w1);
     if (b0 == b1) {
         const R f0 = o0 - R(b0 - l0 + (ORD == 2 ? 1 : 0));
         const R f1 = o1 - R(b1 - l1 + (ORD == 2 ? 1 : 0));
@@ -437,9 +438,11 @@ __device__ __forceinline__ void esirkepov3d_extra(const R *S0x, const R *DSx, co
 // The deposit of one particle, by the lanes of the warp that hold one (`lanes`: their
 // mask, used by the warp vote below).  In 2D3V (x-z plane) Wx = DSx (S0z +
 // DSz/2), Wz = DSz (S0x + DSx/2) and the out-of-plane Jy = f_y' (S0x S0z + DSx S0z / 2 +
-// S0x DSz / 2 + DSx DSz / 3) with f_y' = (q w / dV) v_y; the 2D3V loops skip zero
-// contributions (up to 16 particles per cell contend there).  kNarrow (3D): the window
-// adapts to the particles.  With kLane every lane covers ORD + 1 entries along each axis;
+// S0x DSz / 2 + DSx DSz / 3) with f_y' = (q w / dV) v_y.  kNarrow: the window adapts to the
+// particles; without it (FP64) zero contributions are skipped.  In 2D3V a lane covers ORD + 1
+// entries along each axis and, where its particle changes its nodes, the entries beyond
+// (against the (ORD + 2)-wide window with a test of every value 525 instead of 703 warp
+// instructions for a warp's particles, of 1,480 and 1,800 in all).  In 3D, with kLane every lane covers ORD + 1 entries along each axis;
 // a lane whose particle changes its z nodes adds the entries beyond them along z
 // (esirkepov3d_zextra) and one that changes its x or y nodes those of the ORD + 2 window
 // beyond them along x and y (esirkepov3d_extra), so the other lanes of its warp add none
@@ -448,17 +451,17 @@ __device__ __forceinline__ void esirkepov3d_extra(const R *S0x, const R *DSx, co
 // nodes (one vote per warp), ORD + 2 otherwise, and ORD + 2 along z.
 template <int ND, int ORD, bool kDisp, bool kNarrow, bool kLane, typename R, typename Acc>
 __device__ __forceinline__ void deposit_esirkepov(unsigned lanes, const int l0[3], const R o0[3], const int l1[3], const R o1[3],
-                                                  const R disp[3], R fx, R fy, R fz, int jlo, int jlo_y, int jd0,
+                                                  const int db[3], const R disp[3], R fx, R fy, R fz, int jlo, int jlo_y, int jd0,
                                                   int jd01, int jvol, const Acc &acc)
 {
     constexpr int W = ORD + 2;
     R S0x[W], DSx[W], S0y[W], DSy[W], S0z[W], DSz[W];
     int nwx, nwy = 1, nwz;
-    const int wsx = shape_window<ORD, kDisp>(l0[0], o0[0], l1[0], o1[0], disp[0], S0x, DSx, nwx) - jlo;
-    const int wsz = shape_window<ORD, kDisp>(l0[2], o0[2], l1[2], o1[2], disp[2], S0z, DSz, nwz) - jlo;
+    const int wsx = shape_window<ORD, kDisp>(l0[0], o0[0], l1[0], o1[0], db[0], disp[0], S0x, DSx, nwx) - jlo;
+    const int wsz = shape_window<ORD, kDisp>(l0[2], o0[2], l1[2], o1[2], db[2], disp[2], S0z, DSz, nwz) - jlo;
     const R half = R(0.5), third = R(1.0 / 3.0);
     if (ND == 3) {
-        const int wsy = shape_window<ORD, kDisp>(l0[1], o0[1], l1[1], o1[1], disp[1], S0y, DSy, nwy) - jlo_y;
+        const int wsy = shape_window<ORD, kDisp>(l0[1], o0[1], l1[1], o1[1], db[1], disp[1], S0y, DSy, nwy) - jlo_y;
         const int base = wsx + jd0 * wsy + jd01 * wsz;
         if (kNarrow && kLane) {
             esirkepov3d<ORD + 1, ORD + 1, ORD + 1, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
@@ -474,34 +477,63 @@ __device__ __forceinline__ void deposit_esirkepov(unsigned lanes, const int l0[3
     } else {
         // fy carries the out-of-plane factor (q w / dV) v_y here
         const int base = wsx + jd01 * wsz;
-#pragma unroll
-        for (int k = 0; k < W; ++k) {
-            const R fY = fx * (S0z[k] + half * DSz[k]);
+        // a current entry by its value: Jx at face i of row k, Jz at face k of column i, Jy at
+        // node (i, k)
+        auto jx = [&](int i, int k) {
             R run = R(0);
 #pragma unroll
-            for (int i = 0; i < W - 1; ++i) {
-                run += DSx[i];
-                const R v = fY * run;
-                if (v != R(0)) acc.add(base + i + jd01 * k, v);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-            const R fX = fz * (S0x[i] + half * DSx[i]);
+            for (int m = 0; m <= i; ++m) run += DSx[m];
+            return fx * (S0z[k] + half * DSz[k]) * run;
+        };
+        auto jz = [&](int i, int k) {
             R run = R(0);
 #pragma unroll
-            for (int k = 0; k < W - 1; ++k) {
-                run += DSz[k];
-                const R v = fX * run;
-                if (v != R(0)) acc.add(2 * jvol + base + i + jd01 * k, v);
+            for (int m = 0; m <= k; ++m) run += DSz[m];
+            return fz * (S0x[i] + half * DSx[i]) * run;
+        };
+        auto jy = [&](int i, int k) {
+            return fy * (S0x[i] * S0z[k] + half * (DSx[i] * S0z[k] + S0x[i] * DSz[k]) + third * DSx[i] * DSz[k]);
+        };
+        auto put = [&](int comp, int i, int k, R v) {
+            if (!kNarrow && v == R(0)) return;
+            acc.add(comp * jvol + base + i + jd01 * k, v);
+        };
+        // every lane: the nodes a particle keeps ...
+        constexpr int N = kNarrow ? ORD + 1 : W;
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int i = 0; i < N - 1; ++i) put(0, i, k, jx(i, k));
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int k = 0; k < N - 1; ++k) put(2, i, k, jz(i, k));
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int i = 0; i < N; ++i) put(1, i, k, jy(i, k));
+        // ... and the lanes that change their z or x nodes the row or column beyond them
+        if (kNarrow && nwz > N) {
+#pragma unroll
+            for (int i = 0; i < N - 1; ++i) put(0, i, N, jx(i, N));
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                put(2, i, N - 1, jz(i, N - 1));
+                put(1, i, N, jy(i, N));
             }
         }
+        if (kNarrow && nwx > N) {
 #pragma unroll
-        for (int k = 0; k < W; ++k) {
+            for (int k = 0; k < N; ++k) {
+                put(0, N - 1, k, jx(N - 1, k));
+                put(1, N, k, jy(N, k));
+            }
 #pragma unroll
-            for (int i = 0; i < W; ++i) {
-                const R v = fy * (S0x[i] * S0z[k] + half * (DSx[i] * S0z[k] + S0x[i] * DSz[k]) + third * DSx[i] * DSz[k]);
-                if (v != R(0)) acc.add(jvol + base + i + jd01 * k, v);
+            for (int k = 0; k < N - 1; ++k) put(2, N, k, jz(N, k));
+            if (nwz > N) {
+                put(0, N - 1, N, jx(N - 1, N));
+                put(2, N, N - 1, jz(N, N - 1));
+                put(1, N, N, jy(N, N));
             }
         }
     }
