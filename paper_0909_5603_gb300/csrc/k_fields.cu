@@ -271,9 +271,10 @@ __global__ void __launch_bounds__(256) k_ghost(Launch L, int axis, long long per
 // FP64 field energy sums (1/2) sum (E^2 + B^2) dV per instance.  Each block takes a
 // contiguous range of kEnergyCells cells of the flattened cell space and, for every
 // instance the range meets, sums its part (each cell's E^2 + B^2 in the storage
-// precision, then FP64) and adds it with one atomic: a few thousand atomics per call
-// instead of one per 256 cells, all on the same address.
-constexpr long long kEnergyCells = 8192;
+// precision, then FP64) and adds it with one atomic: a few thousand atomics per call on
+// the same address, and blocks enough for a grid of 10^5 cells (8192 cells a block left 2M
+// cells on 256 blocks: 60 us).
+constexpr long long kEnergyCells = 2048;
 
 // sum of v over the block (every thread gets it)
 __device__ __forceinline__ double block_sum(double v, double *red)
@@ -362,9 +363,10 @@ __global__ void k_dive(InstDev I, double *dense, long long ncell)
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= ncell) return;
     CellPos c;
-    c.i = (int)(g % I.n[0]);
-    c.j = (int)((g / I.n[0]) % I.n[1]);
-    c.k = (int)(g / ((long long)I.n[0] * I.n[1]));
+    const int rq = fast_div((int)g, I.div_n0);
+    c.i = (int)g - rq * I.n[0];
+    c.k = fast_div(rq, I.div_n1);
+    c.j = rq - c.k * I.n[1];
     c.p = (c.i + I.gh[0]) + I.sy * (c.j + I.gh[1]) + I.sz * (c.k + I.gh[2]);
     long long up[3], dn[3];
     neighbour_offsets(I, c, up, dn);
@@ -372,7 +374,7 @@ __global__ void k_dive(InstDev I, double *dense, long long ncell)
     for (int a = 0; a < 3; ++a) {
         if (I.ndim == 2 && a == 1) continue;
         const R *E = (const R *)eb_field(I, a);
-        d += ((double)E[c.p] - (double)E[c.p + dn[a]]) / I.dx[a];
+        d += ((double)E[c.p] - (double)E[c.p + dn[a]]) * I.cd.inv_dx[a];  // (three divisions: 0.14 ms for 2M cells)
     }
     dense[g] = d;
 }

@@ -3,6 +3,8 @@
 // read-out, and the FP64 particle reductions and charge deposit used by the getters.
 #include "k_particles.cuh"
 
+#include <algorithm>
+
 namespace pic {
 
 // Source records of every tile, one warp per tile (tile_sources_warp).
@@ -69,134 +71,175 @@ __global__ void __launch_bounds__(256) k_readout(Launch L, const int *const *sta
 }
 
 // -------------------------------------------------------------------------------------
-// Particle reductions for the diagnostics and the charge density: walk every live
-// particle of the current layout (per tile, the chunks' live prefix: buckets 0..26).
+// Particle reductions of one instance for the diagnostics and the charge density: walk
+// every live particle of the current layout, by chunks (their live prefix: buckets 0..26).
+// Each warp of the launch takes a contiguous range of chunks, whatever tiles they belong
+// to, so that a crowded tile is shared out (one block per 16 tiles left 64^3 cells with 16
+// particles each on 32 blocks: 0.55 ms of a 0.77 ms diagnostics call).
 // -------------------------------------------------------------------------------------
-template <typename R>
-__device__ __forceinline__ void load_particle(const InstDev &I, int lay, int pos, int &cell, R o[3], R u[3], R &w)
+struct ChunkWalk {
+    int c, end;  // chunks c .. end - 1
+    int t;       // the tile of chunk c
+};
+
+__device__ __forceinline__ ChunkWalk warp_chunks(const InstDev &I, int cur)
 {
-    cell = I.cell[lay][pos];
-    o[0] = ((const R *)I.off[lay][0])[pos];
-    o[1] = I.ndim == 3 ? ((const R *)I.off[lay][1])[pos] : R(0);
-    o[2] = ((const R *)I.off[lay][2])[pos];
-    for (int a = 0; a < 3; ++a) u[a] = ((const R *)I.u[lay][a])[pos];
-    w = ((const R *)I.w[lay])[pos];
+    const int lane = threadIdx.x & 31;
+    const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), nw = gridDim.x * (blockDim.x >> 5);
+    const int *base = I.chunk_base[cur];
+    const int nch = base[I.ntiles];
+    ChunkWalk k;
+    k.c = (int)((long long)nch * w / nw);
+    k.end = (int)((long long)nch * (w + 1) / nw);
+    // the last tile whose chunks start at or before c: 32 probes a round
+    int lo = 0;
+    for (int len = I.ntiles; len > 1;) {
+        const int step = (len + 31) / 32;
+        const unsigned m = __ballot_sync(0xffffffffu, lane * step < len && base[lo + lane * step] <= k.c);
+        const int hit = m ? 31 - __clz(m) : 0;
+        lo += hit * step;
+        len = min(step, len - hit * step);
+    }
+    k.t = lo;
+    return k;
 }
 
-// FP64 kinetic energy and charge sums per instance.  Each block takes kSumTiles
-// consecutive tiles of the launch and adds, for every instance they belong to, its part
-// with one pair of atomics (one pair per tile before: tens of thousands on two addresses).
-constexpr int kSumTiles = 16;
+// Buffer position of the first particle of chunk k.c and its live particles; moves k.t on.
+__device__ __forceinline__ int chunk_start(const InstDev &I, int cur, ChunkWalk &k, int &live)
+{
+    const int *base = I.chunk_base[cur];
+    while (base[k.t + 1] <= k.c) ++k.t;
+    live = I.chunk_pre[cur][(long long)k.c * kPre + kDead];
+    return I.seg[cur][k.t] + (k.c - base[k.t]) * I.R;
+}
 
+// FP64 kinetic energy (without the mass) and weight sums, and the live count; one set of
+// atomics per block.
 template <typename R>
-__global__ void __launch_bounds__(256) k_particle_sums(Launch L, double *sums /* 2 per instance */)
+__global__ void __launch_bounds__(256) k_particle_sums(Launch L, double *sums, unsigned long long *n_live)
 {
     __shared__ double s_ke[8], s_q[8];
-    const int g0 = blockIdx.x * kSumTiles, g1 = min(g0 + kSumTiles, L.total_tiles);
-    if (g0 >= g1) return;
-    int ii = find_instance(L.tile_start, L.ninst, g0);
-    for (int lo = g0; lo < g1; ++ii) {
-        const int hi = min(g1, L.tile_start[ii + 1]);
-        const InstDev &I = L.inst[ii];
-        const int cur = *I.cur;
-        // an instance with a device error may hold a step's layout half written: its
-        // chunk records are not read (the read-out reports the error instead)
-        const bool skip = *(volatile const int *)I.err != 0;
-        double ke = 0.0, q = 0.0;
-        for (int g = skip ? hi : lo; g < hi; ++g) {
-            const int t = g - L.tile_start[ii];
-            const int s0 = I.seg[cur][t];
-            const int c0 = I.chunk_base[cur][t], c1 = I.chunk_base[cur][t + 1];
-            for (int c = c0; c < c1; ++c) {
-                const int live = I.chunk_pre[cur][(long long)c * kPre + kDead];
-                const int start = s0 + (c - c0) * I.R;
-                for (int p = threadIdx.x; p < live; p += blockDim.x) {
-                    const int pos = start + p;  // momenta and weight only: half the particle's bytes
-                    R u[3];
-                    for (int a = 0; a < 3; ++a) u[a] = ((const R *)I.u[cur][a])[pos];
-                    const R w = ((const R *)I.w[cur])[pos];
-                    if (sizeof(R) == 8) {
-                        const double g2 = 1.0 + (double)u[0] * u[0] + (double)u[1] * u[1] + (double)u[2] * u[2];
-                        ke += (double)w * I.m * (sqrt(g2) - 1.0);
-                    } else {
-                        // FP32 storage: gamma - 1 = u^2 / (1 + gamma) in FP32 (no cancellation;
-                        // the stored momenta carry FP32 precision anyway), summed in FP64
-                        const float uu = (float)u[0] * (float)u[0] + (float)u[1] * (float)u[1] + (float)u[2] * (float)u[2];
-                        ke += (double)((float)w * (uu / (1.f + sqrtf(1.f + uu)))) * I.m;
-                    }
-                    q += I.q * (double)w;
-                }
+    __shared__ int s_n[8];
+    const InstDev &I = L.inst[0];
+    const int cur = *I.cur;
+    // an instance with a device error may hold a step's layout half written: its chunk
+    // records are not read (the read-out reports the error instead)
+    if (*(volatile const int *)I.err != 0) return;
+    const R *ux = (const R *)I.u[cur][0], *uy = (const R *)I.u[cur][1], *uz = (const R *)I.u[cur][2], *wt = (const R *)I.w[cur];
+    const int lane = threadIdx.x & 31;
+    double ke = 0.0, q = 0.0;
+    int n = 0;
+    for (ChunkWalk k = warp_chunks(I, cur); k.c < k.end; ++k.c) {
+        int live;
+        const int start = chunk_start(I, cur, k, live);
+        n += live;
+#pragma unroll 8
+        for (int p = lane; p < live; p += 32) {
+            const int pos = start + p;  // momenta and weight only: half the particle's bytes
+            const R u0 = ux[pos], u1 = uy[pos], u2 = uz[pos], w = wt[pos];
+            if (sizeof(R) == 8) {
+                const double g2 = 1.0 + (double)u0 * u0 + (double)u1 * u1 + (double)u2 * u2;
+                ke += (double)w * (sqrt(g2) - 1.0);
+            } else {
+                // FP32 storage: gamma - 1 = u^2 / (1 + gamma) in FP32 (no cancellation; the
+                // stored momenta carry FP32 precision anyway), summed in FP64
+                const float uu = (float)u0 * (float)u0 + (float)u1 * (float)u1 + (float)u2 * (float)u2;
+                ke += (double)((float)w * (uu / (1.f + sqrtf(1.f + uu))));
             }
+            q += (double)w;
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            ke += __shfl_down_sync(0xffffffffu, ke, o);
-            q += __shfl_down_sync(0xffffffffu, q, o);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        ke += __shfl_down_sync(0xffffffffu, ke, o);
+        q += __shfl_down_sync(0xffffffffu, q, o);
+    }
+    if (lane == 0) {
+        s_ke[threadIdx.x >> 5] = ke;
+        s_q[threadIdx.x >> 5] = q;
+        s_n[threadIdx.x >> 5] = n;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double a = 0.0, b = 0.0;
+        unsigned long long m = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+            a += s_ke[w];
+            b += s_q[w];
+            m += (unsigned long long)s_n[w];
         }
-        __syncthreads();  // the shared sums of the previous instance are read
-        if ((threadIdx.x & 31) == 0) {
-            s_ke[threadIdx.x >> 5] = ke;
-            s_q[threadIdx.x >> 5] = q;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double a = 0.0, b = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-                a += s_ke[w];
-                b += s_q[w];
-            }
-            if (a != 0.0) atomicAdd(sums + 2 * ii + 0, a);
-            if (b != 0.0) atomicAdd(sums + 2 * ii + 1, b);
-        }
-        lo = hi;
+        if (m == 0) return;
+        atomicAdd(sums + 0, a * I.m);
+        atomicAdd(sums + 1, b * I.q);
+        atomicAdd(n_live, m);
     }
 }
 
-template <int ORD, typename R>
-__global__ void __launch_bounds__(256) k_rho(Launch L, double *rho /* dense n0*n1*n2 per instance 0 */)
+// The diagnostics' integers beside its sums, so that one copy brings all to the host:
+// sums[3] removed particles, sums[4] the error word (as 64-bit integers).
+__global__ void k_diag_words(Launch L, double *sums)
 {
-    const int g = blockIdx.x;
-    const int ii = find_instance(L.tile_start, L.ninst, g);
-    const InstDev &I = L.inst[ii];
-    const int t = g - L.tile_start[ii];
+    const InstDev &I = L.inst[0];
+    unsigned long long *w = (unsigned long long *)sums;
+    w[3] = *I.lost;
+    w[4] = (unsigned long long)*(volatile const int *)I.err;
+}
+
+// Charge density on the nodes: per particle the wrapped node indices and the weights along
+// each axis once (a weight beyond an absorbing face is zero), then products and FP64 atomics.
+template <int ND, int ORD, typename R>
+__global__ void __launch_bounds__(256) k_rho(Launch L, double *rho /* dense n0*n1*n2 of the instance */)
+{
+    const InstDev &I = L.inst[0];
     const int cur = *I.cur;
-    const int s0 = I.seg[cur][t];
-    const int c0 = I.chunk_base[cur][t], c1 = I.chunk_base[cur][t + 1];
-    const double dV = I.dx[0] * I.dx[1] * I.dx[2];
-    for (int c = c0; c < c1; ++c) {
-        const int live = I.chunk_pre[cur][(long long)c * kPre + kDead];
-        const int start = s0 + (c - c0) * I.R;
-        for (int p = threadIdx.x; p < live; p += blockDim.x) {
-            int cell;
-            R o[3], u[3], w;
-            load_particle(I, cur, start + p, cell, o, u, w);
-            const int cc[3] = {cell % I.n[0], (cell / I.n[0]) % I.n[1], cell / (I.n[0] * I.n[1])};
-            double wt[3][ORD + 1];
-            int b[3];
+    const int *cells = I.cell[cur];
+    const R *of[3] = {(const R *)I.off[cur][0], (const R *)I.off[cur][1], (const R *)I.off[cur][2]};
+    const R *wt = (const R *)I.w[cur];
+    const int n[3] = {I.n[0], I.n[1], I.n[2]};
+    const bool per[3] = {I.bc[0] == 0, I.bc[1] == 0, I.bc[2] == 0};
+    const FastDiv d0 = I.div_n0, d1 = I.div_n1;
+    const double qdv = I.q / (I.dx[0] * I.dx[1] * I.dx[2]);
+    const int lane = threadIdx.x & 31;
+    for (ChunkWalk k = warp_chunks(I, cur); k.c < k.end; ++k.c) {
+        int live;
+        const int start = chunk_start(I, cur, k, live);
+        for (int p = lane; p < live; p += 32) {
+            const int pos = start + p;
+            const int c = cells[pos];
+            const int cq = fast_div(c, d0);
+            const int cz = ND == 3 ? fast_div(cq, d1) : cq;
+            const int cc[3] = {c - cq * n[0], ND == 3 ? cq - cz * n[1] : 0, cz};
+            const int st[3] = {1, n[0], n[0] * n[1]};
+            double w[3][ORD + 1];
+            int at[3][ORD + 1];
+#pragma unroll
             for (int a = 0; a < 3; ++a) {
-                if (I.ndim == 2 && a == 1) {
-                    b[a] = 0;
-                    for (int q = 0; q <= ORD; ++q) wt[a][q] = q == 0 ? 1.0 : 0.0;
-                    continue;
-                }
-                b[a] = shape_nodal<ORD, double>(cc[a], (double)o[a], wt[a]);
-            }
-            const double qw = I.q * (double)w / dV;
-            for (int k = 0; k <= ORD; ++k)
-                for (int j = 0; j <= ORD; ++j)
-                    for (int i = 0; i <= ORD; ++i) {
-                        const double v = qw * wt[0][i] * wt[1][j] * wt[2][k];
-                        if (v == 0.0) continue;
-                        int x[3] = {b[0] + i, b[1] + j, b[2] + k};
-                        bool keep = true;
-                        for (int a = 0; a < 3; ++a) {
-                            if (I.ndim == 2 && a == 1) { x[a] = 0; continue; }
-                            if (x[a] < 0 || x[a] >= I.n[a]) {
-                                if (I.bc[a] == 0) x[a] = (x[a] + I.n[a]) % I.n[a];
-                                else keep = false;
-                            }
-                        }
-                        if (keep) atomicAdd(rho + x[0] + (long long)I.n[0] * (x[1] + (long long)I.n[1] * x[2]), v);
+                if (ND == 2 && a == 1) continue;
+                const int b = shape_nodal<ORD, double>(cc[a], (double)of[a][pos], w[a]);
+#pragma unroll
+                for (int m = 0; m <= ORD; ++m) {
+                    int x = b + m;
+                    if (x < 0 || x >= n[a]) {
+                        if (per[a]) x += x < 0 ? n[a] : -n[a];
+                        else x = 0, w[a][m] = 0.0;
                     }
+                    at[a][m] = x * st[a];
+                }
+            }
+            const double qw = qdv * (double)wt[pos];
+#pragma unroll
+            for (int i = 0; i <= ORD; ++i) {
+                const double wi = qw * w[0][i];
+#pragma unroll
+                for (int j = 0; j <= (ND == 3 ? ORD : 0); ++j) {
+                    const double wij = ND == 3 ? wi * w[1][j] : wi;
+                    double *row = rho + at[0][i] + (ND == 3 ? at[1][j] : 0);
+#pragma unroll
+                    for (int m = 0; m <= ORD; ++m) {
+                        const double v = wij * w[2][m];
+                        if (v != 0.0) atomicAdd(row + at[2][m], v);
+                    }
+                }
+            }
         }
     }
 }
@@ -264,38 +307,50 @@ cudaError_t launch_readout(int fp64, const Launch &L, int cap, const int *const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_particle_sums(int fp64, const Launch &L, double *sums, cudaStream_t s)
+// Blocks of the chunk walks: as many as are resident, fewer when there are fewer chunks.
+static unsigned walk_blocks(int chunk_cap)
 {
-    const unsigned nb = (unsigned)((L.total_tiles + kSumTiles - 1) / kSumTiles);
-    if (fp64)
-        k_particle_sums<double><<<nb, 256, 0, s>>>(L, sums);
-    else
-        k_particle_sums<float><<<nb, 256, 0, s>>>(L, sums);
+    return (unsigned)std::max(1, std::min(152 * 8, (chunk_cap + 7) / 8));
+}
+
+cudaError_t launch_particle_sums(int fp64, const Launch &L, int chunk_cap, double *sums, cudaStream_t s)
+{
+    const unsigned nb = walk_blocks(chunk_cap);
+    unsigned long long *n = (unsigned long long *)(sums + 5);
+    if (fp64) k_particle_sums<double><<<nb, 256, 0, s>>>(L, sums, n);
+    else k_particle_sums<float><<<nb, 256, 0, s>>>(L, sums, n);
     return cudaGetLastError();
 }
 
-// Loads the density kernels of one (order, precision) on the current device: CUDA loads
-// kernels lazily, on their first launch or attribute query.
-cudaError_t preload_rho(int order, int fp64)
+cudaError_t launch_diag_words(const Launch &L, double *sums, cudaStream_t s)
+{
+    k_diag_words<<<1, 1, 0, s>>>(L, sums);
+    return cudaGetLastError();
+}
+
+using RhoKernel = void (*)(Launch, double *);
+static RhoKernel rho_kernel(int ndim, int order, int fp64)
+{
+    if (ndim == 3)
+        return order == 1 ? (fp64 ? k_rho<3, 1, double> : k_rho<3, 1, float>) : (fp64 ? k_rho<3, 2, double> : k_rho<3, 2, float>);
+    return order == 1 ? (fp64 ? k_rho<2, 1, double> : k_rho<2, 1, float>) : (fp64 ? k_rho<2, 2, double> : k_rho<2, 2, float>);
+}
+
+// Loads the density kernels of one (dimension, order, precision) on the current device: CUDA
+// loads kernels lazily, on their first launch or attribute query.
+cudaError_t preload_rho(int ndim, int order, int fp64)
 {
     cudaFuncAttributes a;
-    cudaError_t e = order == 1 ? (fp64 ? cudaFuncGetAttributes(&a, k_rho<1, double>) : cudaFuncGetAttributes(&a, k_rho<1, float>))
-                               : (fp64 ? cudaFuncGetAttributes(&a, k_rho<2, double>) : cudaFuncGetAttributes(&a, k_rho<2, float>));
+    cudaError_t e = cudaFuncGetAttributes(&a, rho_kernel(ndim, order, fp64));
     return e == cudaSuccess ? preload_rho_ion() : e;
 }
 
-cudaError_t launch_rho(int order, int fp64, const Launch &L, double *rho, cudaStream_t s)
+cudaError_t launch_rho(int order, int fp64, const Launch &L, const InstDev &I, double *rho, cudaStream_t s)
 {
-    if (order == 1) {
-        if (fp64) k_rho<1, double><<<L.total_tiles, 256, 0, s>>>(L, rho);
-        else k_rho<1, float><<<L.total_tiles, 256, 0, s>>>(L, rho);
-    } else {
-        if (fp64) k_rho<2, double><<<L.total_tiles, 256, 0, s>>>(L, rho);
-        else k_rho<2, float><<<L.total_tiles, 256, 0, s>>>(L, rho);
-    }
+    rho_kernel(I.ndim, order, fp64)<<<walk_blocks(I.chunk_cap), 256, 0, s>>>(L, rho);
     cudaError_t e = cudaGetLastError();
-    // plus the ion background of a lab-frame plasma (no-op without one)
-    return e == cudaSuccess ? launch_rho_ion(L, L.total_cells, rho, s) : e;
+    // plus the ion background of a lab-frame plasma
+    return e == cudaSuccess && I.ion ? launch_rho_ion(L, I, rho, s) : e;
 }
 
 }  // namespace pic

@@ -110,6 +110,7 @@ bool ctx_view(pic_ctx *c, CtxView *v)
 {
     if (!c || !v) return false;
     v->launch = &c->L;
+    v->inst = &c->h;
     v->order = c->order;
     v->fp64 = c->fp64;
     v->ncell = c->ncell;
@@ -570,7 +571,7 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
                cudaMemcpyAsync(c->d_pencil, pencils, sizeof(pencils), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
                prepare_particles(c->ndim, c->order, c->fp64, o.pusher, c->smem) == cudaSuccess &&
                prepare_fields(c->fp64) == cudaSuccess &&
-               noalloc_load_grid(c->order, c->fp64) == cudaSuccess;
+               noalloc_load_grid(c->ndim, c->order, c->fp64) == cudaSuccess;
     if (!okc || upload_inst(c) != PIC_OK) {
         cudaError_t e = cudaGetLastError();
         dfree_all(c);
@@ -1493,25 +1494,47 @@ extern "C" pic_status pic_synchronize(pic_ctx *ctx)
 // ------------------------------------------------------------------------------------
 // getters
 // ------------------------------------------------------------------------------------
+// Components one after the other through the dense scratch into host_out, queued on the
+// stream behind the work in flight with one synchronisation at the end (six components of
+// a 128x128 grid: 320 us with three synchronisations each).  The density walks the
+// particle layout, which a step that ended in a device error may have left half written:
+// such an error is looked for first.
+static pic_status read_fields(pic_ctx *c, const int *comps, int ncomp, double *host_out)
+{
+    const size_t bytes = sizeof(double) * (size_t)c->ncell;
+    cudaStream_t s = c->stream;
+    cudaSetDevice(c->device);
+    for (int i = 0; i < ncomp; ++i)
+        if (comps[i] == PIC_RHO) {
+            const pic_status st = pic_synchronize(c);
+            if (st != PIC_OK) return st;
+            break;
+        }
+    for (int i = 0; i < ncomp; ++i) {
+        if (comps[i] == PIC_RHO) {
+            CUDA_OR_FAIL(c, cudaMemsetAsync(c->d_dense, 0, bytes, s));
+            if (c->loaded) CUDA_OR_FAIL(c, launch_rho(c->order, c->fp64, c->L, c->h, c->d_dense, s));
+        } else if (comps[i] == PIC_DIVE) {
+            CUDA_OR_FAIL(c, launch_dive(c->fp64, c->h, c->d_dense, c->ncell, s));
+        } else {
+            CUDA_OR_FAIL(c, launch_pack(c->fp64, c->h, comps[i], c->last_filtered, c->d_dense, c->ncell, s));
+        }
+        CUDA_OR_FAIL(c, cudaMemcpyAsync(host_out + (size_t)i * c->ncell, c->d_dense, bytes, cudaMemcpyDeviceToHost, s));
+    }
+    int err = 0;
+    CUDA_OR_FAIL(c, cudaMemcpyAsync(&err, c->h.err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CUDA_OR_FAIL(c, cudaStreamSynchronize(s));
+    CUDA_OR_FAIL(c, cudaGetLastError());
+    return device_error_status(c, err);
+}
+
 extern "C" pic_status pic_get_field(pic_ctx *ctx, int comp, double *host_out, size_t count)
 {
     if (!ctx) return PIC_ERR_ARG;
     if (ctx->is_batch) return fail(ctx, PIC_ERR_ARG, "getters take a member, not a batch");
     if (comp < PIC_EX || comp > PIC_DIVE) return fail(ctx, PIC_ERR_ARG, "component %d invalid", comp);
     if (!host_out || count < (size_t)ctx->ncell) return fail(ctx, PIC_ERR_ARG, "need room for %lld values", ctx->ncell);
-    pic_status st = pic_synchronize(ctx);
-    if (st != PIC_OK) return st;
-    if (comp == PIC_RHO) {
-        CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_dense, 0, sizeof(double) * (size_t)ctx->ncell, ctx->stream));
-        if (ctx->loaded) CUDA_OR_FAIL(ctx, launch_rho(ctx->order, ctx->fp64, ctx->L, ctx->d_dense, ctx->stream));
-    } else if (comp == PIC_DIVE) {
-        CUDA_OR_FAIL(ctx, launch_dive(ctx->fp64, ctx->h, ctx->d_dense, ctx->ncell, ctx->stream));
-    } else {
-        CUDA_OR_FAIL(ctx, launch_pack(ctx->fp64, ctx->h, comp, ctx->last_filtered, ctx->d_dense, ctx->ncell, ctx->stream));
-    }
-    CUDA_OR_FAIL(ctx, cudaMemcpyAsync(host_out, ctx->d_dense, sizeof(double) * (size_t)ctx->ncell, cudaMemcpyDeviceToHost, ctx->stream));
-    CUDA_OR_FAIL(ctx, cudaStreamSynchronize(ctx->stream));
-    return check_device_error(ctx);
+    return read_fields(ctx, &comp, 1, host_out);
 }
 
 extern "C" pic_status pic_get_fields(pic_ctx *ctx, const int *comps, int ncomp, double *host_out, size_t count)
@@ -1520,11 +1543,10 @@ extern "C" pic_status pic_get_fields(pic_ctx *ctx, const int *comps, int ncomp, 
     if (ncomp < 1 || !comps) return fail(ctx, PIC_ERR_ARG, "need at least one component");
     if (!host_out || count / (size_t)ncomp < (size_t)ctx->ncell)
         return fail(ctx, PIC_ERR_ARG, "need room for %d x %lld values", ncomp, ctx->ncell);
-    for (int i = 0; i < ncomp; ++i) {
-        const pic_status st = pic_get_field(ctx, comps[i], host_out + (size_t)i * ctx->ncell, (size_t)ctx->ncell);
-        if (st != PIC_OK) return st;
-    }
-    return PIC_OK;
+    if (ctx->is_batch) return fail(ctx, PIC_ERR_ARG, "getters take a member, not a batch");
+    for (int i = 0; i < ncomp; ++i)
+        if (comps[i] < PIC_EX || comps[i] > PIC_DIVE) return fail(ctx, PIC_ERR_ARG, "component %d invalid", comps[i]);
+    return read_fields(ctx, comps, ncomp, host_out);
 }
 
 extern "C" pic_status pic_get_gauss_residual(pic_ctx *ctx, double *max_abs, double *rms)
@@ -1537,7 +1559,7 @@ extern "C" pic_status pic_get_gauss_residual(pic_ctx *ctx, double *max_abs, doub
     if (!rho) return fail(ctx, PIC_ERR_OOM, "no device memory for the charge density");
     cudaStream_t s = ctx->stream;
     cudaError_t e = cudaMemsetAsync(rho, 0, sizeof(double) * (size_t)ctx->ncell, s);
-    if (e == cudaSuccess && ctx->loaded) e = launch_rho(ctx->order, ctx->fp64, ctx->L, rho, s);
+    if (e == cudaSuccess && ctx->loaded) e = launch_rho(ctx->order, ctx->fp64, ctx->L, ctx->h, rho, s);
     if (e == cudaSuccess) e = launch_dive(ctx->fp64, ctx->h, ctx->d_dense, ctx->ncell, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_sums, 0, 2 * sizeof(double), s);
     if (e == cudaSuccess)
@@ -1967,23 +1989,21 @@ extern "C" pic_status pic_get_diagnostics(pic_ctx *ctx, pic_diag *out)
     if (ctx->is_batch) return fail(ctx, PIC_ERR_ARG, "getters take a member, not a batch");
     cudaSetDevice(ctx->device);
     std::memset(out, 0, sizeof(*out));
-    // the reductions, the live count and the read-back queued behind the work in flight,
-    // with one synchronisation; the particle sums skip an instance whose error word is set
-    // (its layout may be half written), and that error is what the call returns
+    // the reductions (with the live count) and one read-back queued behind the work in
+    // flight, with one synchronisation; the particle sums skip an instance whose error word
+    // is set (its layout may be half written), and that error is what the call returns
     cudaStream_t s = ctx->stream;
-    CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_sums, 0, 3 * sizeof(double), s));
-    if (ctx->loaded) CUDA_OR_FAIL(ctx, launch_particle_sums(ctx->fp64, ctx->L, ctx->d_sums, s));
+    double sums[6];
+    CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_sums, 0, sizeof(sums), s));
+    if (ctx->loaded) CUDA_OR_FAIL(ctx, launch_particle_sums(ctx->fp64, ctx->L, ctx->h.chunk_cap, ctx->d_sums, s));
     CUDA_OR_FAIL(ctx, launch_field_energy(ctx->fp64, ctx->L, ctx->d_sums, s));
-    if (ctx->loaded) CUDA_OR_FAIL(ctx, launch_scan(ctx->L, 1, ctx->d_start_ptr, s));
-    double sums[3];
-    unsigned long long lost = 0;
-    int live = 0, err = 0;
+    CUDA_OR_FAIL(ctx, launch_diag_words(ctx->L, ctx->d_sums, s));
     CUDA_OR_FAIL(ctx, cudaMemcpyAsync(sums, ctx->d_sums, sizeof(sums), cudaMemcpyDeviceToHost, s));
-    CUDA_OR_FAIL(ctx, cudaMemcpyAsync(&lost, ctx->h.lost, sizeof(lost), cudaMemcpyDeviceToHost, s));
-    if (ctx->loaded) CUDA_OR_FAIL(ctx, cudaMemcpyAsync(&live, ctx->h.live, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CUDA_OR_FAIL(ctx, cudaMemcpyAsync(&err, ctx->h.err, sizeof(int), cudaMemcpyDeviceToHost, s));
     CUDA_OR_FAIL(ctx, cudaStreamSynchronize(s));
     CUDA_OR_FAIL(ctx, cudaGetLastError());
+    unsigned long long words[3];  // removed, error word, live
+    std::memcpy(words, sums + 3, sizeof(words));
+    const int err = (int)words[1];
     out->error_flags = err;
     pic_status st = device_error_status(ctx, err);
     if (st != PIC_OK) return st;
@@ -1992,8 +2012,8 @@ extern "C" pic_status pic_get_diagnostics(pic_ctx *ctx, pic_diag *out)
     out->kinetic_energy = sums[0];
     out->total_charge = sums[1];
     out->field_energy = sums[2];
-    out->n_particles = live;
-    out->n_lost = (int64_t)lost;
+    out->n_particles = (int64_t)words[2];
+    out->n_lost = (int64_t)words[0];
     return PIC_OK;
 }
 

@@ -73,7 +73,8 @@ cudaError_t launch_plasma_write(int fp64, const InstDev &I, const PlasmaGen &G, 
 cudaError_t launch_j_init_one(int fp64, const Launch &L, const InstDev &h, cudaStream_t s);
 // the same for a batch; ions: some instance has an ion background
 cudaError_t launch_j_init_batch(int fp64, const Launch &L, bool ions, cudaStream_t s);
-cudaError_t launch_rho_ion(const Launch &L, long long ncell, double *rho, cudaStream_t s);
+// I: the instance's host copy
+cudaError_t launch_rho_ion(const Launch &L, const InstDev &I, double *rho, cudaStream_t s);
 // inj: some instance of the launch has a beam injection plane
 // one: for a launch of one instance, its host copy (passed to the kernel by value); null
 // for a batch
@@ -88,8 +89,12 @@ cudaError_t launch_tile_sources(const Launch &L, cudaStream_t s);
 // cap: the particles its buffers hold
 cudaError_t launch_readout(int fp64, const Launch &L, int cap, const int *const *start, int *cell, void *off, void *u,
                            void *w, int *id, cudaStream_t s);
-cudaError_t launch_particle_sums(int fp64, const Launch &L, double *sums, cudaStream_t s);
-cudaError_t launch_rho(int order, int fp64, const Launch &L, double *rho, cudaStream_t s);
+// kinetic energy and charge of one instance into sums[0], sums[1], its live particles into
+// sums[5] (a 64-bit integer), all zero before; chunk_cap: the chunk records its buffers hold
+cudaError_t launch_particle_sums(int fp64, const Launch &L, int chunk_cap, double *sums, cudaStream_t s);
+// removed particles and error word into sums[3], sums[4] (64-bit integers)
+cudaError_t launch_diag_words(const Launch &L, double *sums, cudaStream_t s);
+cudaError_t launch_rho(int order, int fp64, const Launch &L, const InstDev &I, double *rho, cudaStream_t s);
 // ---- persistent batched step (k_persist.cu)
 // sizes of one instance that set its work items per phase
 struct PersistCounts {
@@ -208,8 +213,8 @@ cudaError_t prepare_particles(int ndim, int order, int fp64, int pusher, size_t 
 // Loads, on the current device, the no-allocation charge work grid (pic_get_rho_noalloc)
 // and the density kernels that read-out launches: CUDA loads code and device arrays on
 // first use, so pic_create calls this and the read-out itself never triggers a load.
-cudaError_t noalloc_load_grid(int order, int fp64);
-cudaError_t preload_rho(int order, int fp64);
+cudaError_t noalloc_load_grid(int ndim, int order, int fp64);
+cudaError_t preload_rho(int ndim, int order, int fp64);
 cudaError_t preload_rho_ion();
 cudaError_t launch_field_energy(int fp64, const Launch &L, double *sums, cudaStream_t s);
 cudaError_t launch_pack(int fp64, const InstDev &I, int comp, int filtered, double *dense, long long ncell, cudaStream_t s);
@@ -227,6 +232,7 @@ cudaError_t launch_residual(const double *a, const double *b, long long n, unsig
 // Read-only view of a pic_ctx (defined in pic_api.cu) for entry points in other files.
 struct CtxView {
     const Launch *launch;
+    const InstDev *inst;  // host copy
     int order, fp64;
     long long ncell;
     cudaStream_t stream;

@@ -45,11 +45,11 @@ namespace pic {
 // CUDA loads a module lazily, on the first use of one of its symbols, and loading this
 // one allocates the work grid: pic_create (with its device current) does that first use,
 // and loads the density kernels the read-out launches.
-cudaError_t noalloc_load_grid(int order, int fp64)
+cudaError_t noalloc_load_grid(int ndim, int order, int fp64)
 {
     void *p = nullptr;
     const cudaError_t e = cudaGetSymbolAddress(&p, g_rho_scratch);
-    return e == cudaSuccess ? preload_rho(order, fp64) : e;
+    return e == cudaSuccess ? preload_rho(ndim, order, fp64) : e;
 }
 
 }  // namespace pic
@@ -77,7 +77,7 @@ extern "C" pic_status pic_get_rho_noalloc(pic_ctx *ctx, double *host_out, size_t
     // the array keeps the previous call's contents: clear the part this grid uses
     const size_t bytes = sizeof(double) * (size_t)v.ncell;
     cudaError_t e = cudaMemsetAsync(grid, 0, bytes, v.stream);
-    if (e == cudaSuccess && v.loaded) e = launch_rho(v.order, v.fp64, *v.launch, grid, v.stream);
+    if (e == cudaSuccess && v.loaded) e = launch_rho(v.order, v.fp64, *v.launch, *v.inst, grid, v.stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(host_out, grid, bytes, cudaMemcpyDeviceToHost, v.stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(v.stream);
     if (e != cudaSuccess) {
