@@ -318,30 +318,6 @@ __device__ __forceinline__ R interp(const R *f, int bx, int bxy, int i0, int j0,
     return acc;
 }
 
-// Global index of J tile element e (component stride jst, local x, y, z) after wrapping
-// (periodic) or clipping (absorbing, returns -1) its guard cells; -1 for the padding
-// entries jvol .. jst - 1 of a component.
-__device__ __forceinline__ long long j_global_index(const InstDev &I, const int T0[3], int ND, int e, int jvol, int jst,
-                                                    int &comp)
-{
-    comp = e / jst;
-    const int rem = e - comp * jst;
-    if (rem >= jvol) return -1;
-    const int lx = rem % I.jdim[0];
-    const int ly = (rem / I.jdim[0]) % I.jdim[1];
-    const int lz = rem / (I.jdim[0] * I.jdim[1]);
-    int gidx[3] = {T0[0] + I.jlo + lx, ND == 3 ? T0[1] + I.jlo + ly : 0, T0[2] + I.jlo + lz};
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        if (ND == 2 && a == 1) continue;
-        if (gidx[a] < 0 || gidx[a] >= I.n[a]) {
-            if (I.bc[a] != 0) return -1;
-            gidx[a] += gidx[a] < 0 ? I.n[a] : -I.n[a];
-        }
-    }
-    return (gidx[0] + I.gh[0]) + I.sy * (gidx[1] + I.gh[1]) + I.sz * (gidx[2] + I.gh[2]);
-}
-
 // FP32 tile, after a chunk: T += A * inv[component], A = 0 over the entries this thread
 // owns, 4 at a time (components start on multiples of 4 entries, jst apart; the arrays
 // start 16-byte aligned).
@@ -438,19 +414,6 @@ __device__ __forceinline__ void flush_j_chunk(const InstDev &I, const int T0[3],
     }
 }
 
-__device__ __forceinline__ void flush_j_double(const InstDev &I, const int T0[3], int ND, const double *J, int jvol,
-                                               int jst, int tid, int nt)
-{
-    for (int e = tid; e < 3 * jst; e += nt) {
-        const double v = J[e];
-        if (v == 0.0) continue;
-        int comp;
-        const long long gi = j_global_index(I, T0, ND, e, jvol, jst, comp);
-        if (gi < 0) continue;
-        atomicAdd((double *)I.J[comp] + gi, v);
-    }
-}
-
 // The same table computed by one warp per tile ahead of the particle kernel (no block
 // barriers, at full occupancy), stored as the tile's source record: the particle count,
 // the number of non-empty sub-ranges (-1 when more than kSubCache) and their first slots
@@ -542,7 +505,7 @@ __device__ __forceinline__ void tile_sources_warp(const Launch &L, int g, SrcScr
         if (fits) rec[kRecSlot + written] = slot_run;
         // the parts of the coming phase (the scan has laid out its output)
         const int *cb = I.chunk_base[1 - lay];
-        const int ch = cb[t + 1] - cb[t], m = part_chunks(cb[I.ntiles]);
+        const int ch = cb[t + 1] - cb[t], m = part_chunks(cb[I.ntiles], I.part_min);
         int first = -1;
         if (ch > 2 * m && I.over_max > 0) {
             const int more = (ch + m - 1) / m - 1;
@@ -670,12 +633,10 @@ static __device__ __forceinline__ void close_parts(const InstDev &I, int out, in
 // plane carries none of its code).  I is the instance's entry of the launch's device
 // array, or, for a launch of one instance, a kernel parameter: its fields are then
 // operands from the constant bank, which no store of the kernel can alias, so they are
-// never reloaded after the particle write-out.  LANEWIN: the deposit window per lane
-// (deposit_esirkepov's kLane), taken where the registers allow it (the one-instance
-// kernel).  PARTS: t may be a tile worked on in parts, of which this CTA takes `part`; its
+// never reloaded after the particle write-out.  PARTS: t may be a tile worked on in parts, of which this CTA takes `part`; its
 // chunk records and totals are then relative to the part until the tile's last part to
 // finish adds the earlier parts' totals to them.
-template <int ND, int ORD, typename R, int PUSHER, bool INJ, bool LANEWIN, bool PARTS>
+template <int ND, int ORD, typename R, int PUSHER, bool INJ, bool PARTS>
 __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, const int part)
 {
     constexpr bool kFixed = sizeof(R) == 4;  // FP32: fixed-point chunk accumulator + FP32 tile
@@ -722,15 +683,15 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
 
     // the tile's slots of this CTA: `mine` of them from `first` on (a whole number of chunks)
     const int split = PARTS ? I.split[t] : -1;
-    const int pch = split >= 0 ? part_chunks(I.chunk_base[out][I.ntiles]) : 0;
+    const int pch = split >= 0 ? part_chunks(I.chunk_base[out][I.ntiles], I.part_min) : 0;
     const int first = split >= 0 ? part * pch * kChunk : 0;
     const int mine = split >= 0 ? min(count - first, pch * kChunk) : count;
     const int seg_mine = seg_out + first, chunk_mine = chunk_out + first / kChunk;
 
     // shared-memory carve-up (base rounded up to 128 bytes for TMA): 6 field boxes, then
-    // the J tile: 3 components of jvol cells, jst = jvol rounded up to a multiple of 4 apart,
-    // as FP64 values (FP64 mode) or as the 32-bit integer chunk accumulator A and the FP32
-    // tile T of 3 jst entries each (FP32 mode) -- 8 bytes per entry either way
+    // in FP32 mode the J tile: 3 components of jvol cells, jst = jvol rounded up to a multiple
+    // of 4 apart, as the 32-bit integer chunk accumulator A and the FP32 tile T of 3 jst
+    // entries each
     const int boxn = I.box[0] * I.box[1] * I.box[2];
     const int box_bytes = boxn * (int)sizeof(R);
     const int box_stride = (box_bytes + 127) & ~127;
@@ -742,7 +703,6 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
     const int jv4 = 3 * (jst >> 2);  // J-tile entries in groups of 4
     int *sJA = reinterpret_cast<int *>(sJraw);
     float *sJT = reinterpret_cast<float *>(sJA + 4 * jv4);
-    double *sJD = reinterpret_cast<double *>(sJraw);
 
     if (tid == 0) {
         mbar_init(&bar, 1);
@@ -755,8 +715,9 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
         for (int c = 0; c < 6; ++c)
             tma_load_3d(sbase + c * box_stride, tm + c, x, y, z, &bar);
     }
-    for (int e = tid; e < 2 * jv4; e += kNT)  // A and T (or the FP64 tile)
-        reinterpret_cast<int4 *>(sJraw)[e] = make_int4(0, 0, 0, 0);
+    if constexpr (kFixed)
+        for (int e = tid; e < 2 * jv4; e += kNT)  // A and T
+            reinterpret_cast<int4 *>(sJraw)[e] = make_int4(0, 0, 0, 0);
     if (tid < kBuckets) s_run[tid] = 0;
     // the tile's source table: its precomputed record (one coalesced read), or built here
     // when the record overflowed
@@ -1077,15 +1038,11 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
                 fy = ND == 3 ? -qw * jfy : qw * s_pu[pb][1][dslot];
                 fz = -qw * jfz;
             }
-            const unsigned lanes = __ballot_sync(0xffffffffu, dep);
             if (dep)
-                deposit_esirkepov<ND, ORD, true, true, LANEWIN, R>(lanes, l, o, l1, o1, db, disp, fx * sc[0], fy * sc[1],
-                                                                   fz * sc[2], I.jlo, jlo_y, jd0, jd01, jst,
-                                                                   ChunkAcc{sJA});
+                deposit_esirkepov<ND, ORD, true, R>(l, o, l1, o1, db, disp, fx * sc[0], fy * sc[1], fz * sc[2],
+                                                    ChunkAcc{sJA, I.jlo, jlo_y, jd0, jd01, jst});
         } else {
-            if (have)
-                deposit_esirkepov<ND, ORD, false, false, false, R>(0u, l, o, l1, o1, db, disp, fx, fy, fz, I.jlo, jlo_y, jd0,
-                                                                   jd01, jst, DoubleAcc{sJD});
+            if (have) deposit_esirkepov<ND, ORD, false, R>(l, o, l1, o1, db, disp, fx, fy, fz, GlobalAcc(I, T0));
         }
 
         // ---- stable ranking of the chunk by bucket: order (warp, lane), one barrier per
@@ -1163,10 +1120,7 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
     if (tid == 0 && s_run[kDead] > 0) atomicAdd(I.lost, (unsigned long long)s_run[kDead]);
 
     // ---- flush the J tile
-    if constexpr (kFixed)
-        flush_j_chunk(I, T0, ND, sJA, sJT, jst, inv, warp, lane);
-    else
-        flush_j_double(I, T0, ND, sJD, jvol, jst, tid, kNT);
+    if constexpr (kFixed) flush_j_chunk(I, T0, ND, sJA, sJT, jst, inv, warp, lane);
 
     if (PARTS && split >= 0) close_parts(I, out, t, split, count, pch, chunk_out, S);
 }
@@ -1186,7 +1140,7 @@ template <int ND, int ORD, typename R, int PUSHER, bool INJ>
 __device__ __forceinline__ void particle_tile_of_launch(const Launch &L, const int g)
 {
     const int ii = find_instance(L.tile_start, L.ninst, g);
-    particle_tile<ND, ORD, R, PUSHER, INJ, false, false>(L.inst[ii], g - L.tile_start[ii], 0);
+    particle_tile<ND, ORD, R, PUSHER, INJ, false>(L.inst[ii], g - L.tile_start[ii], 0);
 }
 
 template <int ND, int ORD, typename R, int PUSHER, bool INJ>
@@ -1201,7 +1155,7 @@ __global__ void __launch_bounds__(kNT, particle_blocks<ND, R>()) k_particles(Lau
     const uint64_t *src = reinterpret_cast<const uint64_t *>(L.inst + ii);
     for (int e = threadIdx.x; e < (int)(sizeof(InstDev) / 8); e += kNT) reinterpret_cast<uint64_t *>(&I)[e] = src[e];
     __syncthreads();
-    particle_tile<ND, ORD, R, PUSHER, INJ, false, false>(I, g - L.tile_start[ii], 0);
+    particle_tile<ND, ORD, R, PUSHER, INJ, false>(I, g - L.tile_start[ii], 0);
 }
 
 // a launch of one instance: the instance by value.  The first I.over_max blocks take the
@@ -1218,7 +1172,7 @@ __global__ void __launch_bounds__(kNT, particle_blocks<ND, R>()) k_particles_one
         t = e.x;
         part = e.y;
     }
-    particle_tile<ND, ORD, R, PUSHER, INJ, true, true>(I, t, part);
+    particle_tile<ND, ORD, R, PUSHER, INJ, true>(I, t, part);
 }
 
 }  // namespace pic

@@ -434,12 +434,13 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
     h.jlo = -shape_order;
     for (int a = 0; a < 3; ++a) h.jdim[a] = activeaxis(c->ndim, a) ? ts[a] + (shape_order == 2 ? 5 : 3) : 1;
     const size_t boxb = ((size_t)h.box[0] * h.box[1] * h.box[2] * c->es + 127) / 128 * 128;
-    // 6 field boxes + the J tile at 8 bytes per cell and component (FP64 values, or the
-    // 32-bit chunk accumulator and the FP32 tile in FP32 mode; each component rounded up to
-    // a multiple of 4 entries) + alignment slack
-    c->smem = 128 + 6 * boxb + 3 * (((size_t)h.jdim[0] * h.jdim[1] * h.jdim[2] + 3) / 4 * 4) * 8;
-    if (c->smem > 200 * 1024) {
-        const size_t smem = c->smem;
+    // 6 field boxes + the J tile at 8 bytes per cell and component (the 32-bit chunk
+    // accumulator and the FP32 tile; each component rounded up to a multiple of 4 entries) +
+    // alignment slack.  FP64 mode has no J tile; the limit on the tile counts one for both
+    const size_t jbytes = 3 * (((size_t)h.jdim[0] * h.jdim[1] * h.jdim[2] + 3) / 4 * 4) * 8;
+    c->smem = 128 + 6 * boxb + (c->fp64 ? 0 : jbytes);
+    if (128 + 6 * boxb + jbytes > 200 * 1024) {
+        const size_t smem = 128 + 6 * boxb + jbytes;
         delete c;
         return fail(nullptr, PIC_ERR_ARG, "tile too large: %zu bytes of shared memory per CTA", smem);
     }
@@ -488,6 +489,7 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
         h.E2[a] = F + (size_t)(12 + a) * h.cstride * c->es;
         h.B2[a] = F + (size_t)(15 + a) * h.cstride * c->es;
     }
+    h.part_min = c->fp64 || h.ntiles < kResidentParts ? 1 : 8;
     h.over = (int2 *)parts;
     h.part_tot = parts + 2 * kMaxOver;
     h.split = h.part_tot + kBuckets * kMaxOver;
@@ -777,7 +779,7 @@ static pic_status upload_layout(pic_ctx *c, const std::vector<int> &seg)
     // chunks the buffers hold bound the parts.
     int most = 0;
     for (int t = 0; t < h.ntiles; ++t) most = std::max(most, cbase[t + 1] - cbase[t]);
-    h.over_max = 2 * most > 3 * part_chunks(nchunks) ? std::min(h.chunk_cap / kMinPart, kMaxOver) : 0;
+    h.over_max = 2 * most > 3 * part_chunks(nchunks, h.part_min) ? std::min(h.chunk_cap / h.part_min, kMaxOver) : 0;
     if (nchunks > h.chunk_cap) return fail(c, PIC_ERR_INTERNAL, "chunk capacity");
     std::vector<int> pre((size_t)std::max(nchunks, 1) * kPre, 0), cbv((size_t)std::max(nchunks, 1) * kBuckets, 0);
     for (int t = 0; t < h.ntiles; ++t) {

@@ -171,11 +171,20 @@ __device__ __forceinline__ int shape_window(int l0, R o0, int l1, R o1, int db, 
 // FP32 tile, T += A / scale, A = 0.  The resolution is 2^-22 of the chunk's largest
 // contribution bound per component, comparable with FP32 accumulation of a cell holding
 // a few contributions, and the chunk sums do not depend on the order of the additions.
-// DoubleAcc (FP64 mode): FP64 shared atomics, zero contributions skipped.
+// GlobalAcc (FP64 mode): FP64 reductions straight to the global J, the window's entries
+// wrapped into a periodic box and dropped beyond an absorbing face.  An FP64 add in shared
+// memory is a compare-and-swap loop whose additions run again for every lane that lost the
+// race, on a pipe of two FP64 lanes per SM and clock that bounds this mode; the reductions
+// are formed in L2, beside it (with the window adapted to the particle and fewer FP64 divisions:
+// 48x48x128 cells with 2 particles each 1.69 -> 1.03 ms).
 // ------------------------------------------------------------------------------------
 struct ChunkAcc {
-    static constexpr bool kSkipZero = false;  // 3D: zero adds cost less than the branch
     int *A;
+    int jlo, jlo_y, jd0, jd01, jvol;  // the J tile: origin, strides, component stride
+    __device__ __forceinline__ int place(int wsx, int wsy, int wsz) const
+    {
+        return wsx - jlo + jd0 * (wsy - jlo_y) + jd01 * (wsz - jlo);
+    }
     // adds round(a * b)
     __device__ __forceinline__ void add_prod(int idx, float a, float b) const
     {
@@ -189,22 +198,51 @@ struct ChunkAcc {
     }
 };
 
-struct DoubleAcc {
-    static constexpr bool kSkipZero = true;
-    double *J;
-    __device__ __forceinline__ void add(int idx, double x) const { atomicAdd(J + idx, x); }
-    __device__ __forceinline__ void add_prod(int idx, double a, double b) const { atomicAdd(J + idx, a * b); }
+struct GlobalAcc {
+    // entry (i, j, k) of component c is index i + 4 j + 16 k + 64 c, a constant in the unrolled
+    // loops, so its offset is a sum of three registers
+    static constexpr int jd0 = 4, jd01 = 16, jvol = 64;
+    const InstDev &I;
+    const int *T0;  // the tile's first cell
+    long long zo[4];
+    int yo[4], xo[4];
+    unsigned ok;    // bits i, 4 + j, 8 + k: that node is in the box
+    __device__ __forceinline__ GlobalAcc(const InstDev &inst, const int *t0) : I(inst), T0(t0) {}
+    template <int A>
+    __device__ __forceinline__ int node(int x, int m)
+    {
+        if (x < 0 || x >= I.n[A]) {
+            if (I.bc[A] != 0) return I.gh[A];  // (its bit stays clear)
+            x += x < 0 ? I.n[A] : -I.n[A];
+        }
+        ok |= 1u << (4 * A + m);
+        return x + I.gh[A];
+    }
+    __device__ __forceinline__ int place(int wsx, int wsy, int wsz)
+    {
+        ok = 0;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            xo[m] = node<0>(T0[0] + wsx + m, m);
+            if (I.ndim == 3) yo[m] = (int)I.sy * node<1>(T0[1] + wsy + m, m);
+            else yo[m] = 0, ok |= 1u << (4 + m);
+            zo[m] = I.sz * node<2>(T0[2] + wsz + m, m);
+        }
+        return 0;
+    }
+    __device__ __forceinline__ void add(int idx, double v) const
+    {
+        const int i = idx & 3, j = (idx >> 2) & 3, k = (idx >> 4) & 3, c = idx >> 6;
+        const unsigned need = 1u << i | 16u << j | 256u << k;
+        if ((ok & need) == need) atomicAdd((double *)I.J[c] + zo[k] + yo[j] + xo[i], v);
+    }
+    __device__ __forceinline__ void add_prod(int idx, double a, double b) const { add(idx, a * b); }
 };
 
 template <typename R, typename Acc>
 __device__ __forceinline__ void acc_put(const Acc &acc, int idx, R a, R b)
 {
-    if (Acc::kSkipZero) {
-        const R v = a * b;
-        if (v != R(0)) acc.add(idx, v);
-    } else {
-        acc.add_prod(idx, a, b);
-    }
+    acc.add_prod(idx, a, b);
 }
 
 // ------------------------------------------------------------------------------------
@@ -435,48 +473,34 @@ __device__ __forceinline__ void esirkepov3d_extra(const R *S0x, const R *DSx, co
     }
 }
 
-// The deposit of one particle, by the lanes of the warp that hold one (`lanes`: their
-// mask, used by the warp vote below).  In 2D3V (x-z plane) Wx = DSx (S0z +
-// DSz/2), Wz = DSz (S0x + DSx/2) and the out-of-plane Jy = f_y' (S0x S0z + DSx S0z / 2 +
-// S0x DSz / 2 + DSx DSz / 3) with f_y' = (q w / dV) v_y.  kNarrow: the window adapts to the
-// particles; without it (FP64) zero contributions are skipped.  In 2D3V a lane covers ORD + 1
-// entries along each axis and, where its particle changes its nodes, the entries beyond
-// (against the (ORD + 2)-wide window with a test of every value 525 instead of 703 warp
-// instructions for a warp's particles, of 1,480 and 1,800 in all).  In 3D, with kLane every lane covers ORD + 1 entries along each axis;
-// a lane whose particle changes its z nodes adds the entries beyond them along z
-// (esirkepov3d_zextra) and one that changes its x or y nodes those of the ORD + 2 window
-// beyond them along x and y (esirkepov3d_extra), so the other lanes of its warp add none
-// of those zeros.  Without kLane (fewer registers: the launches over many instances) the
-// warp covers ORD + 1 entries along x and y when none of its particles changes its x or y
-// nodes (one vote per warp), ORD + 2 otherwise, and ORD + 2 along z.
-template <int ND, int ORD, bool kDisp, bool kNarrow, bool kLane, typename R, typename Acc>
-__device__ __forceinline__ void deposit_esirkepov(unsigned lanes, const int l0[3], const R o0[3], const int l1[3], const R o1[3],
-                                                  const int db[3], const R disp[3], R fx, R fy, R fz, int jlo, int jlo_y, int jd0,
-                                                  int jd01, int jvol, const Acc &acc)
+// The deposit of one particle, by the lanes of a warp that hold one.  In 2D3V (x-z plane)
+// Wx = DSx (S0z + DSz/2), Wz = DSz (S0x + DSx/2) and the out-of-plane Jy = f_y' (S0x S0z +
+// DSx S0z / 2 + S0x DSz / 2 + DSx DSz / 3) with f_y' = (q w / dV) v_y.  The window adapts to the
+// particle: every lane covers ORD + 1 entries along each axis, a lane whose particle changes
+// its z nodes adds the entries beyond them along z and one that changes its x or y nodes
+// those of the ORD + 2 window beyond them along x and y, so the other lanes of its warp add
+// none of those zeros.  (2D3V: 525 instead of 703 warp instructions for a warp's particles, of
+// 1,480 and 1,800 in all, against the ORD + 2 window with a test of every value.)
+template <int ND, int ORD, bool kDisp, typename R, typename Acc>
+__device__ __forceinline__ void deposit_esirkepov(const int l0[3], const R o0[3], const int l1[3], const R o1[3],
+                                                  const int db[3], const R disp[3], R fx, R fy, R fz, Acc acc)
 {
-    constexpr int W = ORD + 2;
+    constexpr int W = ORD + 2, N = ORD + 1;
     R S0x[W], DSx[W], S0y[W], DSy[W], S0z[W], DSz[W];
-    int nwx, nwy = 1, nwz;
-    const int wsx = shape_window<ORD, kDisp>(l0[0], o0[0], l1[0], o1[0], db[0], disp[0], S0x, DSx, nwx) - jlo;
-    const int wsz = shape_window<ORD, kDisp>(l0[2], o0[2], l1[2], o1[2], db[2], disp[2], S0z, DSz, nwz) - jlo;
+    int nwx, nwy = 1, nwz, wsy = 0;
+    const int wsx = shape_window<ORD, kDisp>(l0[0], o0[0], l1[0], o1[0], db[0], disp[0], S0x, DSx, nwx);
+    const int wsz = shape_window<ORD, kDisp>(l0[2], o0[2], l1[2], o1[2], db[2], disp[2], S0z, DSz, nwz);
+    if (ND == 3) wsy = shape_window<ORD, kDisp>(l0[1], o0[1], l1[1], o1[1], db[1], disp[1], S0y, DSy, nwy);
+    const int base = acc.place(wsx, wsy, wsz);
+    const int jd0 = acc.jd0, jd01 = acc.jd01, jvol = acc.jvol;
     const R half = R(0.5), third = R(1.0 / 3.0);
     if (ND == 3) {
-        const int wsy = shape_window<ORD, kDisp>(l0[1], o0[1], l1[1], o1[1], db[1], disp[1], S0y, DSy, nwy) - jlo_y;
-        const int base = wsx + jd0 * wsy + jd01 * wsz;
-        if (kNarrow && kLane) {
-            esirkepov3d<ORD + 1, ORD + 1, ORD + 1, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
-            if (nwz > ORD + 1)
-                esirkepov3d_zextra<ORD + 1, W, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
-            if (nwx > ORD + 1 || nwy > ORD + 1)
-                esirkepov3d_extra<ORD + 1, W, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
-        } else if (kNarrow && !__any_sync(lanes, nwx > ORD + 1 || nwy > ORD + 1)) {
-            esirkepov3d<ORD + 1, ORD + 1, W, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
-        } else {
-            esirkepov3d<W, W, W, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
-        }
+        esirkepov3d<N, N, N, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
+        if (nwz > N) esirkepov3d_zextra<N, W, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
+        if (nwx > N || nwy > N)
+            esirkepov3d_extra<N, W, R>(S0x, DSx, S0y, DSy, S0z, DSz, fx, fy, fz, base, jd0, jd01, jvol, acc);
     } else {
         // fy carries the out-of-plane factor (q w / dV) v_y here
-        const int base = wsx + jd01 * wsz;
         // a current entry by its value: Jx at face i of row k, Jz at face k of column i, Jy at
         // node (i, k)
         auto jx = [&](int i, int k) {
@@ -494,12 +518,8 @@ __device__ __forceinline__ void deposit_esirkepov(unsigned lanes, const int l0[3
         auto jy = [&](int i, int k) {
             return fy * (S0x[i] * S0z[k] + half * (DSx[i] * S0z[k] + S0x[i] * DSz[k]) + third * DSx[i] * DSz[k]);
         };
-        auto put = [&](int comp, int i, int k, R v) {
-            if (!kNarrow && v == R(0)) return;
-            acc.add(comp * jvol + base + i + jd01 * k, v);
-        };
+        auto put = [&](int comp, int i, int k, R v) { acc.add(comp * jvol + base + i + jd01 * k, v); };
         // every lane: the nodes a particle keeps ...
-        constexpr int N = kNarrow ? ORD + 1 : W;
 #pragma unroll
         for (int k = 0; k < N; ++k)
 #pragma unroll
@@ -513,7 +533,7 @@ __device__ __forceinline__ void deposit_esirkepov(unsigned lanes, const int l0[3
 #pragma unroll
             for (int i = 0; i < N; ++i) put(1, i, k, jy(i, k));
         // ... and the lanes that change their z or x nodes the row or column beyond them
-        if (kNarrow && nwz > N) {
+        if (nwz > N) {
 #pragma unroll
             for (int i = 0; i < N - 1; ++i) put(0, i, N, jx(i, N));
 #pragma unroll
@@ -522,7 +542,7 @@ __device__ __forceinline__ void deposit_esirkepov(unsigned lanes, const int l0[3
                 put(1, i, N, jy(i, N));
             }
         }
-        if (kNarrow && nwx > N) {
+        if (nwx > N) {
 #pragma unroll
             for (int k = 0; k < N; ++k) {
                 put(0, N - 1, k, jx(N - 1, k));
@@ -590,7 +610,8 @@ __device__ __forceinline__ void push_vay(float u[3], const float E[3], const flo
 __device__ __forceinline__ void push_vay(double u[3], const double E[3], const double B[3], double h)
 {
     const double g = sqrt(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-    const double v0 = u[0] / g, v1 = u[1] / g, v2 = u[2] / g;
+    const double ig = 1.0 / g;  // (one quotient for three: GB300's FP64 pipe bounds this mode)
+    const double v0 = u[0] * ig, v1 = u[1] * ig, v2 = u[2] * ig;
     const double up0 = u[0] + 2.0 * h * E[0] + h * (v1 * B[2] - v2 * B[1]);
     const double up1 = u[1] + 2.0 * h * E[1] + h * (v2 * B[0] - v0 * B[2]);
     const double up2 = u[2] + 2.0 * h * E[2] + h * (v0 * B[1] - v1 * B[0]);
@@ -601,8 +622,8 @@ __device__ __forceinline__ void push_vay(double u[3], const double E[3], const d
     const double q4 = tau2 + ustar * ustar;
     const double root = sqrt(sigma * sigma + 4.0 * q4);
     const double g2 = sigma >= 0.0 ? 0.5 * (sigma + root) : 2.0 * q4 / (root - sigma);
-    const double gn = sqrt(g2);
-    const double s0 = t0 / gn, s1 = t1 / gn, s2 = t2 / gn;
+    const double ign = 1.0 / sqrt(g2);
+    const double s0 = t0 * ign, s1 = t1 * ign, s2 = t2 * ign;
     const double s = 1.0 / (1.0 + s0 * s0 + s1 * s1 + s2 * s2);
     const double upt = up0 * s0 + up1 * s1 + up2 * s2;
     u[0] = s * (up0 + upt * s0 + (up1 * s2 - up2 * s1));

@@ -33,15 +33,17 @@ constexpr int kSrcRec = (kRecPos + kSubCache + 3) / 4 * 4;  // ints per tile
 // tiles: their number is at most total / part_chunks(total) <= kMaxOver = two for each of
 // the 2 x 152 CTAs that are resident, so that the largest part is about half of a CTA's
 // share of the launch: a bunch of 2^20 electrons in 64x64x256 cells, whose fullest tile
-// holds 520 of its 4,500 chunks, is then balanced.  Parts below 8 chunks would spend more on
-// staging the fields and flushing J than on their particles.
+// holds 520 of its 4,500 chunks, is then balanced.  Parts have at least part_min chunks: 8
+// where there are tiles enough for the resident CTAs, as shorter ones would spend more on
+// staging the fields and flushing J than on their particles; 1 where there are not (128x128
+// cells are 64 tiles) and in FP64, where a chunk takes 50 us and its current needs no flush.
 constexpr int kMaxOver = 608;
-constexpr int kMinPart = 8;
+constexpr int kResidentParts = 304;  // 2 CTAs on each of 152 SMs
 
-__host__ __device__ __forceinline__ int part_chunks(int total_chunks)
+__host__ __device__ __forceinline__ int part_chunks(int total_chunks, int part_min)
 {
     const int m = (total_chunks + kMaxOver - 1) / kMaxOver;
-    return m > kMinPart ? m : kMinPart;
+    return m > part_min ? m : part_min;
 }
 
 // Output slots per CTA of the canonical read-out for a buffer of cap particles: a fuller
@@ -147,6 +149,7 @@ struct InstDev {
                         // in parts, its first entry in over
     int *done;          // [ntiles] parts of the tile completed
     int *n_over;        // entries in over
+    int part_min;       // fewest chunks of a part (part_chunks)
     int over_max;       // room in over for the parts of a step: 0 when no tile was near
                         // crowded at the load, and then no tile is split
     int2 *over;         // [kMaxOver] (tile, part) of the parts beyond a tile's first
