@@ -659,17 +659,24 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
     __shared__ __align__(8) unsigned char s_cnt[2][32][kNW];
     __shared__ __align__(16) unsigned s_bmax[3][kNW];  // FP32: per-warp contribution bounds of the chunk
 
-    const int out = *I.cur;  // the scan of this step already flipped the parity
-    const int in = 1 - out;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // the tile's place in either layout and its source record, loaded beside the parity that
+    // says which layout is which: one memory latency instead of three in a row (with the first
+    // particles staged before the wait for the fields, 128x128x1024 stage: 4.20 -> 4.13 ms)
+    const int out = *I.cur;  // the scan of this step already flipped the parity
+    const int seg_a = I.seg[0][t], end_a = I.seg[0][t + 1], chunk_a = I.chunk_base[0][t];
+    const int seg_b = I.seg[1][t], end_b = I.seg[1][t + 1], chunk_b = I.chunk_base[1][t];
+    const int split = PARTS ? I.split[t] : -1;
+    const int rec = tid < kSrcRec ? I.srcrec[(size_t)t * kSrcRec + tid] : 0;
+    const int in = 1 - out;
 
     const int tx = t % I.nt[0];
     const int ty = (t / I.nt[0]) % I.nt[1];
     const int tz = t / (I.nt[0] * I.nt[1]);
     const int T0[3] = {tx * I.ts[0], ty * I.ts[1], tz * I.ts[2]};
-    const int seg_out = I.seg[out][t];
-    const int count = I.seg[out][t + 1] - seg_out;
-    const int chunk_out = I.chunk_base[out][t];
+    const int seg_out = out ? seg_b : seg_a;
+    const int count = (out ? end_b : end_a) - seg_out;
+    const int chunk_out = out ? chunk_b : chunk_a;
 
     if (count == 0) {
         if (tid < kBuckets) I.tot[out][t * kBuckets + tid] = 0;
@@ -682,7 +689,6 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
     }
 
     // the tile's slots of this CTA: `mine` of them from `first` on (a whole number of chunks)
-    const int split = PARTS ? I.split[t] : -1;
     const int pch = split >= 0 ? part_chunks(I.chunk_base[out][I.ntiles], I.part_min) : 0;
     const int first = split >= 0 ? part * pch * kChunk : 0;
     const int mine = split >= 0 ? min(count - first, pch * kChunk) : count;
@@ -721,26 +727,12 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
     if (tid < kBuckets) s_run[tid] = 0;
     // the tile's source table: its precomputed record (one coalesced read), or built here
     // when the record overflowed
-    {
-        const int *rec = I.srcrec + (size_t)t * kSrcRec;
-        if (tid < kSrcRec) {
-            const int v = rec[tid];
-            if (tid == 0) S.count = v;
-            else if (tid == 1) S.nsub = v;
-            else if (tid >= kRecSlot && tid < kRecPos) S.sub_slot[tid - kRecSlot] = v;
-            else if (tid >= kRecPos && tid < kRecPos + kSubCache) S.sub_pos[tid - kRecPos] = v;
-        }
-        __syncthreads();
-        if (S.nsub < 0) build_sources(I, in, tx, ty, tz, first, first + mine, S);  // ends with __syncthreads
-    }
-    const bool ok = mbar_wait_bounded(&bar, 0, kWaitCycles);
-    if (!__syncthreads_and(ok ? 1 : 0)) {
-        if (tid == 0) {
-            atomicOr(I.err, kErrTimeout);
-            mbar_wait_bounded(&bar, 0, kWaitCycles);  // let copies in flight land
-        }
-        return;
-    }
+    if (tid == 0) S.count = rec;
+    else if (tid == 1) S.nsub = rec;
+    else if (tid >= kRecSlot && tid < kRecPos) S.sub_slot[tid - kRecSlot] = rec;
+    else if (tid >= kRecPos && tid < kRecPos + kSubCache) S.sub_pos[tid - kRecPos] = rec;
+    __syncthreads();
+    if (S.nsub < 0) build_sources(I, in, tx, ty, tz, first, first + mine, S);  // ends with __syncthreads
     if (tid == 0 && S.count != count) atomicOr(I.err, kErrInternal);
 
     // per-instance constants in the working precision (host-formed); in FP32 mode the
@@ -792,6 +784,16 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
         return p;
     };
     int pos_next = stage(tid, 0);
+    // the fields have landed (the first particles are on their way meanwhile)
+    const bool ok = mbar_wait_bounded(&bar, 0, kWaitCycles);
+    if (!__syncthreads_and(ok ? 1 : 0)) {
+        if (tid == 0) {
+            atomicOr(I.err, kErrTimeout);
+            mbar_wait_bounded(&bar, 0, kWaitCycles);  // let copies in flight land
+        }
+        cp_async_wait_all();
+        return;
+    }
     float inv[3] = {1.f, 1.f, 1.f};  // FP32: the current chunk's per-component 1 / scale
     // FP32, 2D3V: the deposit's lanes.  The particles of a tile are nearly sorted by cell, so
     // with many particles per cell the lanes of a warp share a few window starts, and shared
