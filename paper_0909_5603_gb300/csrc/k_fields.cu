@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(256) k_filter_axis(Launch L, int axis, const l
 }
 
 template <typename R, int P>
-__global__ void __launch_bounds__(256) k_filter_col(Launch L, int axis, const long long *pencil_start, int src_is_jt)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_filter_col(Launch L, int axis, const long long *pencil_start, int src_is_jt)
 {
     filter_col_block<R, P>(L, axis, pencil_start, src_is_jt, blockIdx.x);
 }
