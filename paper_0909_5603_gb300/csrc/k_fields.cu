@@ -92,14 +92,14 @@ __global__ void __launch_bounds__(256) k_bhalf(Launch L, int damp)
     Bz[p] = bz;
 }
 
-// The fused Yee update, one CTA per tile and z chunk (maxwell_fused_block).  The CTA of an
+// The fused Yee update (maxwell_fused_block).  The CTA of an
 // instance that finishes last switches it to the buffer pair it wrote (every CTA has read
 // the parity by then), so that no launch follows for it.
 template <typename R, int ND>
-__global__ void __launch_bounds__(MxTile<ND>::X * MxTile<ND>::Y, mx_resident<R, ND>())
+__global__ void __launch_bounds__(32 * mx_warps<ND>(), mx_resident<R, ND>())
     k_maxwell_fused(Launch L, const long long *tile_start, int filtered)
 {
-    maxwell_fused_block<R, ND, MxTile<ND>::X, MxTile<ND>::Y>(L, tile_start, filtered, blockIdx.x, 0, true);
+    maxwell_fused_block<R, ND, mx_warps<ND>()>(L, tile_start, filtered, blockIdx.x, 0, true);
     __syncthreads();
     if (threadIdx.x == 0) {
         const int ii = find_instance_ll(tile_start, L.ninst, blockIdx.x);
@@ -408,14 +408,13 @@ template <typename R, int ND>
 static cudaError_t maxwell_fused_attr()
 {
     return cudaFuncSetAttribute(k_maxwell_fused<R, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)maxwell_fused_smem<R, ND, MxTile<ND>::X, MxTile<ND>::Y>());
+                                (int)maxwell_fused_smem<R, ND, mx_warps<ND>()>());
 }
 
 template <typename R, int ND>
 static void maxwell_fused_t(const Launch &L, const long long *tile_start, unsigned nb, int filtered, cudaStream_t s)
 {
-    constexpr int X = MxTile<ND>::X, Y = MxTile<ND>::Y;
-    k_maxwell_fused<R, ND><<<nb, X * Y, maxwell_fused_smem<R, ND, X, Y>(), s>>>(L, tile_start, filtered);
+    k_maxwell_fused<R, ND><<<nb, 32 * mx_warps<ND>(), maxwell_fused_smem<R, ND, mx_warps<ND>()>(), s>>>(L, tile_start, filtered);
 }
 
 cudaError_t launch_maxwell_fused(int fp64, int ndim, const Launch &L, const long long *tile_start, long long ntiles,

@@ -63,24 +63,52 @@ __device__ __forceinline__ R damp_factor(const InstDev &I, const CellPos &c)
 // flips after the last CTA), so no CTA overwrites a value that a neighbouring CTA still
 // reads.  A cell near a periodic face is also stored at its images in the ghost layers
 // beyond the opposite faces (what the gather's TMA boxes read there), instead of one ghost
-// copy launch per periodic axis.  A CTA takes an x-y tile of TX x TY columns (one thread
-// each) and marches
-// along z through a chunk of tz planes, keeping in shared memory E^n of three planes on
-// the tile widened by [-1, +2] in x and y, B^{n+1/2} of three planes on [-1, +1] and
-// E^{n+1} of two planes on [0, +1].  For the output plane k, between two barriers:
-//   B^{n+1/2}(k+2) = B^n - dt/2 curl E^n        (E^n of planes k+2, k+3)
-//   E^{n+1}(k+1)  = f (E^n + dt (curl B^{n+1/2} - J))   (B^{n+1/2} of planes k, k+1)
-// and after the second:
-//   B^{n+1}(k)    = f (B^{n+1/2} - dt/2 curl E^{n+1})   (E^{n+1} of planes k, k+1)
-// with the loads of the next plane issued one plane ahead.  Outside an absorbing box
-// every field is zero; periodic axes wrap.  Each value is formed by the same expression
-// as in k_bhalf / k_efull; the in-plane offsets of a thread's cells are computed once.
-template <typename R, int ND, int X, int Y>
+// copy launch per periodic axis.
+//
+// A warp is one row of 32 columns along x, a thread one column, and the block marches
+// along z through a chunk of tz planes.  In 3D its NW warps are NW rows along y; the outer
+// column and rows (one below, two above) only feed their neighbours, so a block puts out
+// 29 x (NW - 3) columns.  In 2D3V every warp marches alone through its own strip and chunk.  At
+// plane i a thread forms, of its own column,
+//   B^{n+1/2}(i+2) = B^n - dt/2 curl E^n            (E^n of planes i+2, i+3)
+//   E^{n+1}(i+1)  = f (E^n + dt (curl B^{n+1/2} - J))  (B^{n+1/2} of planes i, i+1)
+//   B^{n+1}(i)    = f (B^{n+1/2} - dt/2 curl E^{n+1})  (E^{n+1} of planes i, i+1)
+// with the planes in registers, the x neighbours by shuffles and only the y neighbours
+// through shared memory, all of them formed at earlier planes: one block barrier per plane
+// (none in 2D3V).  The planes to come are copied (cp.async) into a ring of kMxAhead planes in
+// shared memory, every thread its own column, so their latency costs no registers.
+// Outside an absorbing box every field is zero; periodic axes wrap.  Each value is formed
+// by the same expression as in k_bhalf / k_efull.
+//
+// It is bound by instruction issue (67 %) together with the latency of each plane's chain.
+// Against a thread per column of 32 x 8 with all neighbours in shared memory, two barriers
+// and the next plane's loads in registers, per step: 128x128x1024 380 -> 344 us (1.0 GB, 44 %
+// of the copy rate), 64^3 periodic 37 -> 24, 32x32x256 29 -> 23, 48x48x128 FP64 90 -> 75,
+// 128x128 2D3V 18 -> 9.4, a batch of 32 2D3V instances 108 -> 40 us.
+constexpr int kMxCols = 29;  // columns along x that a warp puts out
+
+template <typename R>
+__host__ __device__ constexpr int mx_ahead()
+{
+    return sizeof(R) == 4 ? 4 : 3;
+}
+
+// the ring (nine components a plane) and, in 3D, rows of y neighbours: two planes of six
+// components
+template <typename R, int ND, int NW>
 constexpr size_t maxwell_fused_smem()
 {
-    constexpr int HY = ND == 3 ? 1 : 0;
-    constexpr size_t NE = (size_t)(X + 3) * (Y + 3 * HY), NB = (size_t)(X + 2) * (Y + 2 * HY), NQ = (size_t)(X + 1) * (Y + HY);
-    return sizeof(R) * 3 * (3 * NE + 3 * NB + 2 * NQ);
+    return sizeof(R) * 32 * NW * (9 * mx_ahead<R>() + (ND == 3 ? 2 * 6 : 0));
+}
+
+// cp.async of one value, or a zero
+template <typename R>
+__device__ __forceinline__ void mx_copy(R *dst, const R *src, bool ok)
+{
+    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(d), "l"(src), "n"(sizeof(R)),
+                 "r"(ok ? (int)sizeof(R) : 0)
+                 : "memory");
 }
 
 // index along one axis of the cell at q: false outside an absorbing box; wrapped on a
@@ -96,34 +124,40 @@ __device__ __forceinline__ bool mx_axis(int q, int n, int bc, int &w)
     return true;
 }
 
-// Block g of the launch's tiles (tile_start: the instances' first tiles), by TX x TY threads.
+// Block g of the launch's tiles (tile_start: the instances' first tiles), by NW warps.
 // tz: planes per chunk (0: the instance's own, mx_planes).  images: also store the periodic
 // images of the cells.
-template <typename R, int ND, int TX, int TY>
+template <typename R, int ND, int NW>
 __device__ __forceinline__ void maxwell_fused_block(const Launch &L, const long long *tile_start, int filtered,
                                                     const long long g, int tz, bool images)
 {
-    constexpr int NT = TX * TY;
-    constexpr int HY = ND == 3 ? 1 : 0;
-    constexpr int EX = TX + 3, NE = EX * (TY + 3 * HY);  // E^n region: [-1, +2]
-    constexpr int BX = TX + 2, NB = BX * (TY + 2 * HY);  // B^{n+1/2} region: [-1, +1]
-    constexpr int QX = TX + 1, NQ = QX * (TY + HY);      // E^{n+1} region: [0, +1]
-    static_assert(NE <= 2 * NT && NB <= 2 * NT && NQ <= 2 * NT, "two region cells per thread");
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int TY = NW - 3, NT = 32 * NW;
     extern __shared__ __align__(16) unsigned char msm[];
-    R *sE = (R *)msm;     // [3 planes][3 comps][NE]
-    R *sH = sE + 9 * NE;  // [3][3][NB]
-    R *sQ = sH + 9 * NB;  // [2][3][NQ]
+    constexpr int D = mx_ahead<R>();
+    R *ring = (R *)msm;         // [plane % D][E of the plane, B of the one before, J of the one before that][thread]
+    R *sm = ring + 9 * D * NT;  // [plane parity][Ex Ez Bx Bz Ex' Ez'][row][32]
     if (g >= tile_start[L.ninst]) return;
     const int ii = find_instance_ll(tile_start, L.ninst, g);
     const InstDev &I = L.inst[ii];
     const int n0 = I.n[0], n1 = I.n[1], n2 = I.n[2];
-    const int ntx = (n0 + TX - 1) / TX, nty = (n1 + TY - 1) / TY;
-    long long r = g - tile_start[ii];
-    const int x0 = (int)(r % ntx) * TX;
-    r /= ntx;
-    const int y0 = (int)(r % nty) * TY;
+    // (the shuffle tells the compiler that the warp's number, and with it its planes, is the
+    // same in all lanes)
+    const int lane = threadIdx.x & 31, row = __shfl_sync(kAll, (int)(threadIdx.x >> 5), 0);
     if (tz == 0) tz = I.mx_planes;
-    const int z0 = (int)(r / nty) * tz;
+    const int ntx = (n0 + kMxCols - 1) / kMxCols;
+    long long r = g - tile_start[ii];
+    if (ND == 2) r = r * NW + row;  // this warp's strip and chunk
+    const int x0 = (int)(r % ntx) * kMxCols;
+    r /= ntx;
+    int y0 = 0;
+    if (ND == 3) {
+        const int nty = (n1 + TY - 1) / TY;
+        y0 = (int)(r % nty) * TY;
+        r /= nty;
+    }
+    const int z0 = (int)r * tz;
+    if (z0 >= n2) return;  // (2D3V: a warp beyond the last strip)
     const int z1 = min(z0 + tz, n2);
     const int par = *(volatile const int *)I.fpar;
     // the components of each field are cstride elements apart
@@ -136,227 +170,184 @@ __device__ __forceinline__ void maxwell_fused_block(const Launch &L, const long 
     const R h = K.half_dt, dt = K.dt;
     const R ix = K.inv_dx[0], iy = K.inv_dx[1], iz = K.inv_dx[2];
     const R *dampx = (const R *)I.damp[0], *dampy = (const R *)I.damp[1], *dampz = (const R *)I.damp[2];
-    const int tid = threadIdx.x;
-    // in-plane padded offset of the cell at (x0 + dx, y0 + dy), false outside the box;
-    // fxy: its x and y damping factors multiplied in the order of damp_factor
-    auto inplane = [&](int dx_, int dy_, int &off, R &fxy) -> bool {
-        int x, y = 0;
-        bool ok = mx_axis(x0 + dx_, n0, I.bc[0], x);
-        if (ND == 3) ok = ok && mx_axis(y0 + dy_, n1, I.bc[1], y);
-        off = (x + I.gh[0]) + I.sy * (y + I.gh[1]);  // < 2^31: one plane
-        fxy = R(1);
-        if (ok && dampx) fxy *= dampx[x];
-        if (ok && ND == 3 && dampy) fxy *= dampy[y];
-        return ok;
+    // this thread's column: its padded in-plane offset, whether it lies in the box, its x
+    // and y damping factors multiplied in the order of damp_factor
+    const int xc = x0 - 1 + lane, yc = ND == 3 ? y0 - 1 + row : 0;
+    int x = 0, y = 0;
+    bool in = mx_axis(xc, n0, I.bc[0], x);
+    if (ND == 3) in = mx_axis(yc, n1, I.bc[1], y) && in;
+    const unsigned off = (unsigned)(x + I.gh[0]) + (unsigned)I.sy * (unsigned)(y + I.gh[1]);  // < 2^31: one plane
+    R fxy = R(1);
+    if (in && dampx) fxy *= dampx[x];
+    if (in && ND == 3 && dampy) fxy *= dampy[y];
+    // whether it is put out here, and where its images lie in the ghost layers of periodic
+    // axes: bit 0 (1) of mx when x is within the ghost width of the lower (upper) face, my for y
+    const bool tok = lane >= 1 && lane <= kMxCols && xc < n0 && (ND == 2 || (row >= 1 && row <= TY && yc < n1));
+    const int mx = images && I.bc[0] == 0 ? (xc < I.gh[0] ? 1 : 0) | (xc >= n0 - I.gh[0] ? 2 : 0) : 0;
+    const int my = ND == 3 && images && I.bc[1] == 0 ? (yc < I.gh[1] ? 1 : 0) | (yc >= n1 - I.gh[1] ? 2 : 0) : 0;
+    // what the planes need of the instance, kept in registers (its device copy would be read
+    // again after every store)
+    const bool per2 = I.bc[2] == 0, zimg = images && per2;
+    const long long sy = I.sy, sz = I.sz;
+    const int gh2 = I.gh[2];
+    // z: padded offset of plane k (-1 <= k <= n2 + 2: at most one wrap), false outside an
+    // absorbing box
+    auto zplane = [&](int k, long long &zo) -> bool {
+        const int z = k < 0 ? k + n2 : k >= n2 ? k - n2 : k;
+        zo = sz * (long long)(z + gh2);
+        return per2 || z == k;
     };
-    int eoff[2], boff[2], qoff[2], toff;
-    bool eok[2], bok[2], qok[2], tok;
-    R qf[2], tf, unused;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int e = tid + NT * j, b = tid + NT * j, q = tid + NT * j;
-        eok[j] = e < NE && inplane(e % EX - 1, e / EX - HY, eoff[j], unused);
-        bok[j] = b < NB && inplane(b % BX - 1, b / BX - HY, boff[j], unused);
-        qok[j] = q < NQ && inplane(q % QX, q / QX, qoff[j], qf[j]);
-    }
-    const int tx = tid % TX, ty = tid / TX;
-    tok = x0 + tx < n0 && y0 + ty < n1 && inplane(tx, ty, toff, tf);
-    // the images of this column in the ghost layers of periodic axes: bit 0 (1) of mx when x
-    // is within the ghost width of the lower (upper) face, my for y
-    const int mx = images && I.bc[0] == 0 ? (x0 + tx < I.gh[0] ? 1 : 0) | (x0 + tx >= n0 - I.gh[0] ? 2 : 0) : 0;
-    const int my = ND == 3 && images && I.bc[1] == 0 ? (y0 + ty < I.gh[1] ? 1 : 0) | (y0 + ty >= n1 - I.gh[1] ? 2 : 0) : 0;
-    const bool zimg = images && I.bc[2] == 0;
-    // z: padded plane offset of plane k, false outside an absorbing box
-    auto zplane = [&](int k, long long &zo, R &fz) -> bool {
-        int z;
-        const bool ok = mx_axis(k, n2, I.bc[2], z);
-        zo = I.sz * (long long)(z + I.gh[2]);
-        fz = (ok && dampz) ? dampz[z] : R(1);
-        return ok;
+    // plane n of the ring: E^n(n), B^n(n-1), J(n-2), as far as the chunk needs them
+    auto fetch = [&](int n) {
+        R *d = ring + (unsigned)(n - z0) % D * 9 * NT + threadIdx.x;
+        auto copy3 = [&](const R *F, int k, R *to, bool wanted) {
+            if (!wanted) return;
+            long long zo;
+            const bool ok = zplane(k, zo) && in;
+            const R *plane = F + zo;  // (off lies in the plane, whether copied or not)
+            mx_copy(to, plane + off, ok);
+            mx_copy(to + NT, plane + cs + off, ok);
+            mx_copy(to + 2 * NT, plane + 2 * cs + off, ok);
+        };
+        copy3(Ein, n, d, n <= z1 + 2);
+        copy3(Bin, n - 1, d + 3 * NT, n - 1 <= z1);
+        copy3(Jin, n - 2, d + 6 * NT, n - 2 >= z0 && n - 2 <= z1);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    auto slot3 = [](int k) { return ((k % 3) + 3) % 3; };
-    // global loads of one plane for this thread's cells of a region
-    auto load3 = [&](const R *F, const int *off, const bool *ok, int k, R (&v)[2][3]) {
-        long long zo;
-        R fz;
-        const bool zk = zplane(k, zo, fz);
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) v[j][c] = (zk && ok[j]) ? F[c * cs + off[j] + zo] : R(0);
-    };
-    auto storeE = [&](int k, const R (&v)[2][3]) {
-        R *d = sE + slot3(k) * 3 * NE;
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-            if (tid + NT * j < NE)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) d[c * NE + tid + NT * j] = v[j][c];
-    };
-    // B^{n+1/2}(k) from E^n of planes k, k+1 and B^n(k) (bv)
-    auto makeH = [&](int k, const R (&bv)[2][3]) {
-        long long zo;
-        R fz;
-        const bool zk = zplane(k, zo, fz);
-        const R *E0 = sE + slot3(k) * 3 * NE, *E1 = sE + slot3(k + 1) * 3 * NE;
-        R *H = sH + slot3(k) * 3 * NB;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int b = tid + NT * j;
-            if (b >= NB) continue;
-            R hb[3] = {R(0), R(0), R(0)};
-            if (zk && bok[j]) {
-                const int e = b % BX + EX * (b / BX);
-                const R ex = E0[e], ey = E0[NE + e], ez = E0[2 * NE + e];
-                R dEz_dy = R(0), dEx_dy = R(0);
-                const R dEy_dz = (E1[NE + e] - ey) * iz;
-                const R dEx_dz = (E1[e] - ex) * iz;
-                const R dEz_dx = (E0[2 * NE + e + 1] - ez) * ix;
-                const R dEy_dx = (E0[NE + e + 1] - ey) * ix;
-                if (ND == 3) {
-                    dEz_dy = (E0[2 * NE + e + EX] - ez) * iy;
-                    dEx_dy = (E0[e + EX] - ex) * iy;
-                }
-                hb[0] = bv[j][0] - h * (dEz_dy - dEy_dz);
-                hb[1] = bv[j][1] - h * (dEx_dz - dEz_dx);
-                hb[2] = bv[j][2] - h * (dEy_dx - dEx_dy);
-            }
-#pragma unroll
-            for (int c = 0; c < 3; ++c) H[c * NB + b] = hb[c];
-        }
-    };
-    // E^{n+1}(k) from B^{n+1/2} of planes k-1, k, E^n(k) and J(k) (jv)
-    auto makeQ = [&](int k, const R (&jv)[2][3]) {
-        long long zo;
-        R fz;
-        const bool zk = zplane(k, zo, fz);
-        const R *H1 = sH + slot3(k) * 3 * NB, *H0 = sH + slot3(k - 1) * 3 * NB;
-        const R *E0 = sE + slot3(k) * 3 * NE;
-        R *Q = sQ + (k & 1) * 3 * NQ;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int q = tid + NT * j;
-            if (q >= NQ) continue;
-            R en[3] = {R(0), R(0), R(0)};
-            if (zk && qok[j]) {
-                const int qx = q % QX, qy = q / QX;
-                const int b = (qx + 1) + BX * (qy + HY), e = (qx + 1) + EX * (qy + HY);
-                const R bx = H1[b], by = H1[NB + b], bz = H1[2 * NB + b];
-                R dBz_dy = R(0), dBx_dy = R(0);
-                const R dBy_dz = (by - H0[NB + b]) * iz, dBx_dz = (bx - H0[b]) * iz;
-                const R dBz_dx = (bz - H1[2 * NB + b - 1]) * ix, dBy_dx = (by - H1[NB + b - 1]) * ix;
-                if (ND == 3) {
-                    dBz_dy = (bz - H1[2 * NB + b - BX]) * iy;
-                    dBx_dy = (bx - H1[b - BX]) * iy;
-                }
-                const R f = dampz ? qf[j] * fz : qf[j];
-                en[0] = f * (E0[e] + dt * ((dBz_dy - dBy_dz) - jv[j][0]));
-                en[1] = f * (E0[NE + e] + dt * ((dBx_dz - dBz_dx) - jv[j][1]));
-                en[2] = f * (E0[2 * NE + e] + dt * ((dBy_dx - dBx_dy) - jv[j][2]));
-            }
-#pragma unroll
-            for (int c = 0; c < 3; ++c) Q[c * NQ + q] = en[c];
-        }
-    };
-    // B^{n+1}(k) on the tile from B^{n+1/2}(k), E^{n+1} of planes k, k+1; stores both
-    auto emit = [&](int k) {
-        if (!tok) return;
-        long long zo;
-        R fz;
-        zplane(k, zo, fz);
-        const R *Q0 = sQ + (k & 1) * 3 * NQ, *Q1 = sQ + ((k + 1) & 1) * 3 * NQ;
-        const R *H = sH + slot3(k) * 3 * NB;
-        const int q = tx + QX * ty, b = (tx + 1) + BX * (ty + HY);
-        const R ex = Q0[q], ey = Q0[NQ + q], ez = Q0[2 * NQ + q];
-        R dEz_dy = R(0), dEx_dy = R(0);
-        const R dEy_dz = (Q1[NQ + q] - ey) * iz;
-        const R dEx_dz = (Q1[q] - ex) * iz;
-        const R dEz_dx = (Q0[2 * NQ + q + 1] - ez) * ix;
-        const R dEy_dx = (Q0[NQ + q + 1] - ey) * ix;
-        if (ND == 3) {
-            dEz_dy = (Q0[2 * NQ + q + QX] - ez) * iy;
-            dEx_dy = (Q0[q + QX] - ex) * iy;
-        }
-        R bx = H[b] - h * (dEz_dy - dEy_dz);
-        R by = H[NB + b] - h * (dEx_dz - dEz_dx);
-        R bz = H[2 * NB + b] - h * (dEy_dx - dEx_dy);
-        const R f = dampz ? tf * fz : tf;
-        bx *= f;
-        by *= f;
-        bz *= f;
-        const long long p = toff + zo;
-        Bout[p] = bx;
-        Bout[cs + p] = by;
-        Bout[2 * cs + p] = bz;
-        Eout[p] = ex;
-        Eout[cs + p] = ey;
-        Eout[2 * cs + p] = ez;
-        const int mz = zimg ? (k < I.gh[2] ? 1 : 0) | (k >= n2 - I.gh[2] ? 2 : 0) : 0;
-        if (mx | my | mz) {
-            // every combination of staying (0), + n (1) and - n (2) along the three axes
-#pragma unroll 1
-            for (int m = 1; m < 27; ++m) {
-                const int ax = m % 3, ay = (m / 3) % 3, az = m / 9;
-                if ((ax && !(mx & ax)) || (ay && !(my & ay)) || (az && !(mz & az))) continue;
-                const long long s = p + (ax == 1 ? n0 : ax == 2 ? -n0 : 0) +
-                                    I.sy * (long long)(ay == 1 ? n1 : ay == 2 ? -n1 : 0) +
-                                    I.sz * (long long)(az == 1 ? n2 : az == 2 ? -n2 : 0);
-                Bout[s] = bx;
-                Bout[cs + s] = by;
-                Bout[2 * cs + s] = bz;
-                Eout[s] = ex;
-                Eout[cs + s] = ey;
-                Eout[2 * cs + s] = ez;
-            }
-        }
-    };
+    const int at = threadIdx.x, up = min(row + 1, NW - 1) * 32 + lane, dn = max(row - 1, 0) * 32 + lane;
 
-    R vE[2][3], cB[2][3], cJ[2][3], nB[2][3], nJ[2][3];
-    // prologue: E^n of planes z0-1 .. z0+2, B^{n+1/2} of z0-1 .. z0+1, E^{n+1} of z0
-    load3(Ein, eoff, eok, z0 - 1, vE);
-    storeE(z0 - 1, vE);
-    load3(Ein, eoff, eok, z0, vE);
-    storeE(z0, vE);
-    load3(Ein, eoff, eok, z0 + 1, vE);
-    storeE(z0 + 1, vE);
-    load3(Bin, boff, bok, z0 - 1, cB);
-    load3(Bin, boff, bok, z0, nB);
-    load3(Jin, qoff, qok, z0, cJ);
-    __syncthreads();
-    makeH(z0 - 1, cB);
-    makeH(z0, nB);
-    __syncthreads();
-    makeQ(z0, cJ);
-    __syncthreads();
-    load3(Ein, eoff, eok, z0 + 2, vE);
-    storeE(z0 + 2, vE);  // in the slot of plane z0 - 1
-    load3(Bin, boff, bok, z0 + 1, cB);
-    __syncthreads();
-    makeH(z0 + 1, cB);   // the third slot
-    // one plane ahead: E^n(z0+3), B^n(z0+2), J(z0+1)
-    load3(Ein, eoff, eok, z0 + 3, vE);
-    load3(Bin, boff, bok, z0 + 2, cB);
-    load3(Jin, qoff, qok, z0 + 1, cJ);
-#pragma unroll 1
-    for (int k = z0; k < z1; ++k) {
-        storeE(k + 3, vE);  // in the slot of plane k
-        // the next plane's loads, in flight through this plane's arithmetic
-        load3(Ein, eoff, eok, k + 4, vE);
-        load3(Bin, boff, bok, k + 3, nB);
-        load3(Jin, qoff, qok, k + 2, nJ);
-        __syncthreads();
-        makeH(k + 2, cB);  // in the slot of plane k - 1
-        makeQ(k + 1, cJ);  // in the slot of plane k - 1
-        __syncthreads();
-        emit(k);
+    R e1[3] = {}, e2[3], h0[3] = {}, h1[3] = {}, q0[3] = {}, f0 = R(1);
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
+    for (int n = 0; n < D; ++n) fetch(z0 + n);
+    {
+        long long zo;
+        const bool ok = zplane(z0 - 1, zo) && in;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) e2[c] = ok ? (Ein + c * cs + zo)[off] : R(0);
+    }
+    if (ND == 3) {
+        R *s = sm + ((z0 - 3) & 1) * 6 * NT;
+        s[at] = e2[0];
+        s[NT + at] = e2[2];
+        __syncthreads();
+    }
+#pragma unroll 1
+    for (int i = z0 - 3; i < z1; ++i) {
+        const R *s = sm + (i & 1) * 6 * NT;
+        R *t = sm + ((i + 1) & 1) * 6 * NT;
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 1) : "memory");
+        R e3[3], b2[3], j1[3];
+        {
+            const R *d = ring + (unsigned)(i + 3 - z0) % D * 9 * NT + threadIdx.x;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                cB[j][c] = nB[j][c];
-                cJ[j][c] = nJ[j][c];
+                e3[c] = d[c * NT];
+                b2[c] = d[(3 + c) * NT];
+                j1[c] = d[(6 + c) * NT];
             }
+        }
+        fetch(i + 3 + D);  // in the place of the plane just taken
+        long long zo;
+        R h2[3] = {R(0), R(0), R(0)}, q1[3] = {R(0), R(0), R(0)}, f1 = fxy;
+        if (i + 2 <= z1) {
+            const R ex = e2[0], ey = e2[1], ez = e2[2];
+            R dEz_dy = R(0), dEx_dy = R(0);
+            const R dEy_dz = (e3[1] - ey) * iz;
+            const R dEx_dz = (e3[0] - ex) * iz;
+            const R dEz_dx = (__shfl_down_sync(kAll, ez, 1) - ez) * ix;
+            const R dEy_dx = (__shfl_down_sync(kAll, ey, 1) - ey) * ix;
+            if (ND == 3) {
+                dEz_dy = (s[NT + up] - ez) * iy;
+                dEx_dy = (s[up] - ex) * iy;
+            }
+            if (zplane(i + 2, zo) && in) {
+                h2[0] = b2[0] - h * (dEz_dy - dEy_dz);
+                h2[1] = b2[1] - h * (dEx_dz - dEz_dx);
+                h2[2] = b2[2] - h * (dEy_dx - dEx_dy);
+            }
+        }
+        if (i + 1 >= z0) {
+            const R bx = h1[0], by = h1[1], bz = h1[2];
+            R dBz_dy = R(0), dBx_dy = R(0);
+            const R dBy_dz = (by - h0[1]) * iz, dBx_dz = (bx - h0[0]) * iz;
+            const R dBz_dx = (bz - __shfl_up_sync(kAll, bz, 1)) * ix, dBy_dx = (by - __shfl_up_sync(kAll, by, 1)) * ix;
+            if (ND == 3) {
+                dBz_dy = (bz - s[3 * NT + dn]) * iy;
+                dBx_dy = (bx - s[2 * NT + dn]) * iy;
+            }
+            if (zplane(i + 1, zo) && in) {
+                const R f = dampz ? fxy * dampz[i + 1] : fxy;  // (an axis with a layer does not wrap)
+                f1 = f;
+                q1[0] = f * (e1[0] + dt * ((dBz_dy - dBy_dz) - j1[0]));
+                q1[1] = f * (e1[1] + dt * ((dBx_dz - dBz_dx) - j1[1]));
+                q1[2] = f * (e1[2] + dt * ((dBy_dx - dBx_dy) - j1[2]));
+            }
+        }
+        if (i >= z0) {
+            const R ex = q0[0], ey = q0[1], ez = q0[2];
+            R dEz_dy = R(0), dEx_dy = R(0);
+            const R dEy_dz = (q1[1] - ey) * iz;
+            const R dEx_dz = (q1[0] - ex) * iz;
+            const R dEz_dx = (__shfl_down_sync(kAll, ez, 1) - ez) * ix;
+            const R dEy_dx = (__shfl_down_sync(kAll, ey, 1) - ey) * ix;
+            if (ND == 3) {
+                dEz_dy = (s[5 * NT + up] - ez) * iy;
+                dEx_dy = (s[4 * NT + up] - ex) * iy;
+            }
+            if (tok) {
+                zo = sz * (long long)(i + gh2);
+                R bx = h0[0] - h * (dEz_dy - dEy_dz);
+                R by = h0[1] - h * (dEx_dz - dEz_dx);
+                R bz = h0[2] - h * (dEy_dx - dEx_dy);
+                bx *= f0;
+                by *= f0;
+                bz *= f0;
+                auto store = [&](long long p, unsigned o) {  // p the same in the whole warp
+                    (Bout + p)[o] = bx;
+                    (Bout + cs + p)[o] = by;
+                    (Bout + 2 * cs + p)[o] = bz;
+                    (Eout + p)[o] = ex;
+                    (Eout + cs + p)[o] = ey;
+                    (Eout + 2 * cs + p)[o] = ez;
+                };
+                // the cell (0) and its images + n (1) and - n (2): along z and y the same for
+                // the whole warp, along x for the lanes near a face
+                const int mz = zimg ? (i < gh2 ? 1 : 0) | (i >= n2 - gh2 ? 2 : 0) : 0;
+#pragma unroll 1
+                for (int az = 0; az <= mz; ++az) {
+                    if (az && !(mz & az)) continue;
+                    const long long pz = zo + sz * (long long)(az == 1 ? n2 : az == 2 ? -n2 : 0);
+#pragma unroll 1
+                    for (int ay = 0; ay <= my; ++ay) {
+                        if (ay && !(my & ay)) continue;
+                        const long long p = pz + sy * (long long)(ay == 1 ? n1 : ay == 2 ? -n1 : 0);
+                        store(p, off);
+                        if (mx & 1) store(p, off + (unsigned)n0);
+                        if (mx & 2) store(p, off - (unsigned)n0);
+                    }
+                }
+            }
+        }
+        if (ND == 3) {
+            t[at] = e3[0];
+            t[NT + at] = e3[2];
+            t[2 * NT + at] = h2[0];
+            t[3 * NT + at] = h2[2];
+            t[4 * NT + at] = q1[0];
+            t[5 * NT + at] = q1[2];
+            __syncthreads();
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            e1[c] = e2[c];
+            e2[c] = e3[c];
+            h0[c] = h1[c];
+            h1[c] = h2[c];
+            q0[c] = q1[c];
+        }
+        f0 = f1;
     }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");  // (only empty groups are left)
 }
 
 // Binomial filter along one axis, all passes at once.  The x, y and z operators (each

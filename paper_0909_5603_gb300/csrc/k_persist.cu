@@ -94,15 +94,11 @@ __device__ __noinline__ void particle_item(const Launch &L, int g)
 }
 
 constexpr int kPersistPlanes = 32;  // planes of a fused Yee item
-template <int ND>
-struct PersistMx {  // columns of a fused Yee item, one per thread of the CTA
-    static constexpr int X = ND == 3 ? 32 : kNT, Y = ND == 3 ? 8 : 1;
-};
 
 template <int ND>
 __device__ __noinline__ void maxwell_item(const Launch &L, const long long *mx_start, int filtered, long long g)
 {
-    maxwell_fused_block<float, ND, PersistMx<ND>::X, PersistMx<ND>::Y>(L, mx_start, filtered, g, kPersistPlanes, false);
+    maxwell_fused_block<float, ND, kNW>(L, mx_start, filtered, g, kPersistPlanes, false);
 }
 
 __device__ __noinline__ void filter_any(const Launch &L, const long long *pen, int axis, int src_is_jt, long long g,
@@ -265,8 +261,7 @@ size_t persist_smem(int ndim, size_t particle_smem)
 {
     // the particle phase's dynamic shared memory, or the largest scratch of another phase
     size_t m = particle_smem;
-    m = std::max(m, ndim == 3 ? maxwell_fused_smem<float, 3, PersistMx<3>::X, PersistMx<3>::Y>()
-                              : maxwell_fused_smem<float, 2, PersistMx<2>::X, PersistMx<2>::Y>());
+    m = std::max(m, ndim == 3 ? maxwell_fused_smem<float, 3, kNW>() : maxwell_fused_smem<float, 2, kNW>());
     m = std::max(m, sizeof(float) * 8 * 3 * (size_t)(kPencil + 2 * 4) + 128);
     m = std::max(m, sizeof(SrcScratch) * 8 + 128);
     m = std::max(m, sizeof(int) * 66 + 128);
@@ -298,8 +293,7 @@ cudaError_t PersistPlan::build(int ndim, const std::vector<PersistCounts> &inst,
             case kPhParticles: c = k.ntiles; break;
             case kPhFilterX: case kPhFilterY: case kPhFilterZ: c = k.pencils[p - kPhFilterX]; break;
             case kPhMaxwell:
-                c = ndim == 3 ? maxwell_tiles(k.n, PersistMx<3>::X, PersistMx<3>::Y, kPersistPlanes)
-                              : maxwell_tiles(k.n, PersistMx<2>::X, PersistMx<2>::Y, kPersistPlanes);
+                c = maxwell_tiles(k.n, ndim, kPersistPlanes, kNW);
                 break;
             case kPhGhostX: case kPhGhostY: case kPhGhostZ: c = (k.ghost[p - kPhGhostX] + kGhostElems - 1) / kGhostElems; break;
             default: c = 1;

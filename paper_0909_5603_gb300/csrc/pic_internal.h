@@ -130,37 +130,29 @@ cudaError_t persist_blocks_per_sm(int ndim, int order, size_t smem, int *bps);
 
 // opt-in to the shared memory of the fused Yee update (once per device and precision)
 cudaError_t prepare_fields(int fp64);
-// Columns of a block of the fused Yee update, and the blocks of an SM: 32 x 8 columns in
-// 3D; in 2D3V 64, so that a narrow grid fills its blocks and several small blocks hide one
-// another's barriers (128 x 128 cells, FP32: 46 us with one block of 256 columns per 32
-// planes).
+// Warps of a block of the fused Yee update (maxwell_fused_block), and its blocks per SM: 16
+// rows put out 13 (8 would put out 5); in 2D3V the warps are independent
 template <int ND>
-struct MxTile;
-template <>
-struct MxTile<3> {
-    static constexpr int X = 32, Y = 8;
-};
-template <>
-struct MxTile<2> {
-    static constexpr int X = 64, Y = 1;
-};
+__host__ __device__ constexpr int mx_warps()
+{
+    return ND == 3 ? 16 : 4;
+}
 template <typename R, int ND>
 constexpr int mx_resident()
 {
-    return ND == 3 ? (sizeof(R) == 4 ? 3 : 2) : (sizeof(R) == 4 ? 12 : 7);
+    return ND == 3 ? (sizeof(R) == 4 ? 2 : 1) : (sizeof(R) == 4 ? 8 : 4);
 }
 // the whole Yee update of the step (Yee solver, no antenna) with its periodic images in one
 // launch over maxwell_tiles() tiles per instance; each instance ends on the E / B buffer
 // pair it wrote
 cudaError_t launch_maxwell_fused(int fp64, int ndim, const Launch &L, const long long *tile_start, long long ntiles,
                                  int filtered, cudaStream_t s);
-inline long long maxwell_tiles(const int n[3], int x, int y, int planes)
+// (warps 0: those of the per-phase launch)
+inline long long maxwell_tiles(const int n[3], int ndim, int planes, int warps = 0)
 {
-    return (long long)((n[0] + x - 1) / x) * ((n[1] + y - 1) / y) * ((n[2] + planes - 1) / planes);
-}
-inline long long maxwell_tiles(const int n[3], int ndim, int planes)
-{
-    return ndim == 3 ? maxwell_tiles(n, MxTile<3>::X, MxTile<3>::Y, planes) : maxwell_tiles(n, MxTile<2>::X, MxTile<2>::Y, planes);
+    if (warps == 0) warps = ndim == 3 ? mx_warps<3>() : mx_warps<2>();
+    const long long strips = (n[0] + 28) / 29, chunks = (n[2] + planes - 1) / planes;
+    return ndim == 3 ? strips * ((n[1] + warps - 4) / (warps - 3)) * chunks : (strips * chunks + warps - 1) / warps;
 }
 // Planes per z chunk for a launch over `count` instances of n[i] cells.  A block works
 // through its planes one after the other behind a prologue of about four, so the launch
