@@ -247,17 +247,17 @@ __global__ void __launch_bounds__(256) k_rho(Launch L, double *rho /* dense n0*n
 // -------------------------------------------------------------------------------------
 // Host-side launchers (called from pic_api.cu).
 // -------------------------------------------------------------------------------------
-cudaError_t dispatch_particles_f32(int ndim, int order, int pusher, const Launch *L, const InstDev *one, size_t smem,
+cudaError_t dispatch_particles_f32(int ndim, int order, int pusher, const Launch *L, const OneInst *one, size_t smem,
                                    cudaStream_t s);
-cudaError_t dispatch_particles_f64(int ndim, int order, int pusher, const Launch *L, const InstDev *one, size_t smem,
+cudaError_t dispatch_particles_f64(int ndim, int order, int pusher, const Launch *L, const OneInst *one, size_t smem,
                                    cudaStream_t s);
-cudaError_t dispatch_particles_f32_inj(int ndim, int order, int pusher, const Launch *L, const InstDev *one, size_t smem,
+cudaError_t dispatch_particles_f32_inj(int ndim, int order, int pusher, const Launch *L, const OneInst *one, size_t smem,
                                    cudaStream_t s);
-cudaError_t dispatch_particles_f64_inj(int ndim, int order, int pusher, const Launch *L, const InstDev *one, size_t smem,
+cudaError_t dispatch_particles_f64_inj(int ndim, int order, int pusher, const Launch *L, const OneInst *one, size_t smem,
                                    cudaStream_t s);
 
 static cudaError_t dispatch_particles(int ndim, int order, int fp64, int pusher, bool inj, const Launch *L,
-                                      const InstDev *one, size_t smem, cudaStream_t s)
+                                      const OneInst *one, size_t smem, cudaStream_t s)
 {
     if (fp64)
         return inj ? dispatch_particles_f64_inj(ndim, order, pusher, L, one, smem, s)
@@ -266,7 +266,7 @@ static cudaError_t dispatch_particles(int ndim, int order, int fp64, int pusher,
                : dispatch_particles_f32(ndim, order, pusher, L, one, smem, s);
 }
 
-cudaError_t launch_particles(int ndim, int order, int fp64, int pusher, bool inj, const Launch &L, const InstDev *one,
+cudaError_t launch_particles(int ndim, int order, int fp64, int pusher, bool inj, const Launch &L, const OneInst *one,
                              size_t smem, cudaStream_t s)
 {
     return dispatch_particles(ndim, order, fp64, pusher, inj, &L, one, smem, s);

@@ -329,6 +329,7 @@ __device__ __forceinline__ void fold_chunk(int *A, float *T, int jst, const floa
     for (int e = tid; e < n4; e += nt) {
         const float s = e >= q2 ? inv[2] : e >= q1 ? inv[1] : inv[0];
         const int4 a = A4[e];
+        if ((a.x | a.y | a.z | a.w) == 0) continue;  // (a chunk touches a few of the tile's planes)
         float4 t = T4[e];
         t.x = __fmaf_rn((float)a.x, s, t.x);
         t.y = __fmaf_rn((float)a.y, s, t.y);
@@ -637,7 +638,7 @@ static __device__ __forceinline__ void close_parts(const InstDev &I, int out, in
 // chunk records and totals are then relative to the part until the tile's last part to
 // finish adds the earlier parts' totals to them.
 template <int ND, int ORD, typename R, int PUSHER, bool INJ, bool PARTS>
-__device__ __forceinline__ void particle_tile(const InstDev &I, const int t, const int part)
+__device__ __forceinline__ void particle_tile(const InstDev &I, const CUtensorMap *tmaps, const int t, const int part)
 {
     constexpr bool kFixed = sizeof(R) == 4;  // FP32: fixed-point chunk accumulator + FP32 tile
     extern __shared__ __align__(128) unsigned char smem[];
@@ -668,11 +669,13 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
     const int seg_b = I.seg[1][t], end_b = I.seg[1][t + 1], chunk_b = I.chunk_base[1][t];
     const int split = PARTS ? I.split[t] : -1;
     const int rec = tid < kSrcRec ? I.srcrec[(size_t)t * kSrcRec + tid] : 0;
+    const int fpar = tid == 0 ? *(volatile const int *)I.fpar : 0;  // the current E / B buffer
     const int in = 1 - out;
 
-    const int tx = t % I.nt[0];
-    const int ty = (t / I.nt[0]) % I.nt[1];
-    const int tz = t / (I.nt[0] * I.nt[1]);
+    const int tyz = fast_div(t, I.div_nt0);
+    const int tx = t - tyz * I.nt[0];
+    const int tz = fast_div(tyz, I.div_nt1);
+    const int ty = tyz - tz * I.nt[1];
     const int T0[3] = {tx * I.ts[0], ty * I.ts[1], tz * I.ts[2]};
     const int seg_out = out ? seg_b : seg_a;
     const int count = (out ? end_b : end_a) - seg_out;
@@ -712,8 +715,9 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const int t, con
 
     if (tid == 0) {
         mbar_init(&bar, 1);
-        const CUtensorMap *tm = I.tmap + 6 * *(volatile const int *)I.fpar;  // the current E / B buffer
-        for (int c = 0; c < 6; ++c) tmap_acquire(tm + c);
+        const CUtensorMap *tm = tmaps + 6 * fpar;
+        if (!PARTS)  // (a launch of one instance has them among its parameters)
+            for (int c = 0; c < 6; ++c) tmap_acquire(tm + c);
         mbar_expect_tx(&bar, 6u * (uint32_t)box_bytes);
         const int x = T0[0] + I.box_lo[0] + I.gh[0];
         const int y = T0[1] + I.box_lo[1] + I.gh[1];
@@ -1142,7 +1146,7 @@ template <int ND, int ORD, typename R, int PUSHER, bool INJ>
 __device__ __forceinline__ void particle_tile_of_launch(const Launch &L, const int g)
 {
     const int ii = find_instance(L.tile_start, L.ninst, g);
-    particle_tile<ND, ORD, R, PUSHER, INJ, false>(L.inst[ii], g - L.tile_start[ii], 0);
+    particle_tile<ND, ORD, R, PUSHER, INJ, false>(L.inst[ii], L.inst[ii].tmap, g - L.tile_start[ii], 0);
 }
 
 template <int ND, int ORD, typename R, int PUSHER, bool INJ>
@@ -1157,7 +1161,7 @@ __global__ void __launch_bounds__(kNT, particle_blocks<ND, R>()) k_particles(Lau
     const uint64_t *src = reinterpret_cast<const uint64_t *>(L.inst + ii);
     for (int e = threadIdx.x; e < (int)(sizeof(InstDev) / 8); e += kNT) reinterpret_cast<uint64_t *>(&I)[e] = src[e];
     __syncthreads();
-    particle_tile<ND, ORD, R, PUSHER, INJ, false>(I, g - L.tile_start[ii], 0);
+    particle_tile<ND, ORD, R, PUSHER, INJ, false>(I, I.tmap, g - L.tile_start[ii], 0);
 }
 
 // a launch of one instance: the instance by value.  The first I.over_max blocks take the
@@ -1165,8 +1169,9 @@ __global__ void __launch_bounds__(kNT, particle_blocks<ND, R>()) k_particles(Lau
 // others one tile each.  (A bunch of 2^20 electrons in 64x64x256 cells, 133,000 of them in
 // one tile: 0.19 ms instead of the 1.14 ms that one CTA needs for that tile.)
 template <int ND, int ORD, typename R, int PUSHER, bool INJ>
-__global__ void __launch_bounds__(kNT, particle_blocks<ND, R>()) k_particles_one(const __grid_constant__ InstDev I)
+__global__ void __launch_bounds__(kNT, particle_blocks<ND, R>()) k_particles_one(const __grid_constant__ OneInst P)
 {
+    const InstDev &I = P.I;
     int t = (int)blockIdx.x - I.over_max, part = 0;
     if (t < 0) {
         if ((int)blockIdx.x >= *I.n_over) return;
@@ -1174,7 +1179,7 @@ __global__ void __launch_bounds__(kNT, particle_blocks<ND, R>()) k_particles_one
         t = e.x;
         part = e.y;
     }
-    particle_tile<ND, ORD, R, PUSHER, INJ, true>(I, t, part);
+    particle_tile<ND, ORD, R, PUSHER, INJ, true>(I, P.tmap, t, part);
 }
 
 }  // namespace pic

@@ -9,7 +9,7 @@ namespace pic {
 // one: the instance of a one-instance launch (host copy, identical to the launch's device
 // entry), passed by value; null for a batch
 template <int ND, int ORD, typename R, int PUSHER, bool INJ>
-static cudaError_t launch_particles_t(const Launch *L, const InstDev *one, size_t smem, cudaStream_t s)
+static cudaError_t launch_particles_t(const Launch *L, const OneInst *one, size_t smem, cudaStream_t s)
 {
     auto k = k_particles<ND, ORD, R, PUSHER, INJ>;
     auto k1 = k_particles_one<ND, ORD, R, PUSHER, INJ>;
@@ -18,14 +18,14 @@ static cudaError_t launch_particles_t(const Launch *L, const InstDev *one, size_
         return e == cudaSuccess ? cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : e;
     }
     if (one && L->ninst == 1)
-        k1<<<L->total_tiles + one->over_max, kNT, smem, s>>>(*one);
+        k1<<<L->total_tiles + one->I.over_max, kNT, smem, s>>>(*one);
     else
         k<<<L->total_tiles, kNT, smem, s>>>(*L);
     return cudaGetLastError();
 }
 
 template <typename R, bool INJ>
-static cudaError_t dispatch_particles_t(int ndim, int order, int pusher, const Launch *L, const InstDev *one, size_t smem,
+static cudaError_t dispatch_particles_t(int ndim, int order, int pusher, const Launch *L, const OneInst *one, size_t smem,
                                         cudaStream_t s)
 {
 #define PIC_DISPATCH(ND, ORD, P) \

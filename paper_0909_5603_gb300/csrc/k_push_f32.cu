@@ -3,7 +3,7 @@
 
 namespace pic {
 
-cudaError_t dispatch_particles_f32(int ndim, int order, int pusher, const Launch *L, const InstDev *one, size_t smem,
+cudaError_t dispatch_particles_f32(int ndim, int order, int pusher, const Launch *L, const OneInst *one, size_t smem,
                                      cudaStream_t s)
 {
     return dispatch_particles_t<float, false>(ndim, order, pusher, L, one, smem, s);

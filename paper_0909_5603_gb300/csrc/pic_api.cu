@@ -44,6 +44,7 @@ struct pic_ctx {
     cudaStream_t stream = nullptr;
     // device views
     InstDev h{};
+    CUtensorMap maps[12];  // host copy of h.tmap
     InstDev *d_inst = nullptr;
     int *d_tile_start = nullptr;
     long long *d_cell_start = nullptr;
@@ -430,6 +431,8 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
     }
     h.div_n0 = make_fastdiv(c->n[0]);
     h.div_n1 = make_fastdiv(c->n[1]);
+    h.div_nt0 = make_fastdiv(h.nt[0]);
+    h.div_nt1 = make_fastdiv(h.nt[1]);
     for (int a = 0; a < 3; ++a) c->fd_ts[a] = make_fastdiv(h.ts[a]);
     h.jlo = -shape_order;
     for (int a = 0; a < 3; ++a) h.jdim[a] = activeaxis(c->ndim, a) ? ts[a] + (shape_order == 2 ? 5 : 3) : 1;
@@ -546,7 +549,7 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
     }
 
     pic_status st = PIC_OK;
-    CUtensorMap maps[12];
+    CUtensorMap *maps = c->maps;
     if ((st = encode_tmaps(c, maps)) != PIC_OK) {
         std::string e = c->err;
         dfree_all(c);
@@ -566,7 +569,7 @@ extern "C" pic_status pic_create(const pic_grid *grid, const double dx[3], doubl
                cudaMemsetAsync(parts, 0, sizeof(int) * ((size_t)(2 + kBuckets) * kMaxOver + 2 * (size_t)h.ntiles + 1), c->stream) ==
                    cudaSuccess &&
                cudaMemsetAsync(tiles, 0, sizeof(int) * (size_t)(4 * nt1 + 2 * h.ntiles * kBuckets + h.ntiles), c->stream) == cudaSuccess &&
-               cudaMemcpyAsync(tm, maps, sizeof(maps), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
+               cudaMemcpyAsync(tm, maps, sizeof(c->maps), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
                cudaMemcpyAsync(c->d_tile_start, tstart, sizeof(tstart), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
                cudaMemcpyAsync(c->d_cell_start, cstart, sizeof(cstart), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
                cudaMemcpyAsync(c->d_start_ptr, &dptr_start, sizeof(int *), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
@@ -1278,7 +1281,10 @@ static pic_status enqueue_step(pic_ctx *c, int mask)
         tm.begin(0);
         bool inj = c->h.inj_id0 != INT_MAX;
         for (auto m : c->members) inj = inj || m->h.inj_id0 != INT_MAX;
-        CUDA_OR_FAIL(c, launch_particles(c->ndim, c->order, fp64, c->opt.pusher, inj, L, c->is_batch ? nullptr : &c->h,
+        OneInst one;
+        one.I = c->h;
+        std::memcpy(one.tmap, c->maps, sizeof(one.tmap));
+        CUDA_OR_FAIL(c, launch_particles(c->ndim, c->order, fp64, c->opt.pusher, inj, L, c->is_batch ? nullptr : &one,
                                          c->smem, c->stream));
         tm.end(0);
         launches += 3;

@@ -164,6 +164,7 @@ struct InstDev {
     const void *damp[3];      // absorbing-layer factor per cell index along each axis
                               // (working precision; null on periodic / inactive axes)
     FastDiv div_n0, div_n1;   // cell index -> (i, j, k)
+    FastDiv div_nt0, div_nt1; // tile index -> tile coordinates
     // ion background of a lab-frame plasma load: lab-stationary ions, i.e. in this frame
     // a rigid density gamma_b n0 p(gamma_b (z + beta_b t)) of charge -q on [0, Lz) at t = 0
     int ion;            // 0: none
@@ -185,6 +186,13 @@ struct InstDev {
     int box_lo[3];      // box origin relative to the tile origin (cells, <= 0)
     int jlo;            // J tile origin relative to the tile origin (-1 or -2)
     int jdim[3];        // J tile extents
+};
+
+// What a launch of one instance passes by value: the instance and its 12 tensor maps (as
+// I.tmap), which among a kernel's parameters need no acquire fence before use.
+struct OneInst {
+    CUtensorMap tmap[12];
+    InstDev I;
 };
 
 template <typename R>

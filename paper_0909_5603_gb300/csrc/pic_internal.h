@@ -78,7 +78,7 @@ cudaError_t launch_rho_ion(const Launch &L, const InstDev &I, double *rho, cudaS
 // inj: some instance of the launch has a beam injection plane
 // one: for a launch of one instance, its host copy (passed to the kernel by value); null
 // for a batch
-cudaError_t launch_particles(int ndim, int order, int fp64, int pusher, bool inj, const Launch &L, const InstDev *one,
+cudaError_t launch_particles(int ndim, int order, int fp64, int pusher, bool inj, const Launch &L, const OneInst *one,
                              size_t smem, cudaStream_t s);
 int particle_chunk();
 int particle_threads();
