@@ -669,7 +669,7 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const CUtensorMa
     const int seg_b = I.seg[1][t], end_b = I.seg[1][t + 1], chunk_b = I.chunk_base[1][t];
     const int split = PARTS ? I.split[t] : -1;
     const int rec = tid < kSrcRec ? I.srcrec[(size_t)t * kSrcRec + tid] : 0;
-    const int fpar = tid == 0 ? *(volatile const int *)I.fpar : 0;  // the current E / B buffer
+    const int fpar = warp == 0 ? *(volatile const int *)I.fpar : 0;  // the current E / B buffer
     const int in = 1 - out;
 
     const int tyz = fast_div(t, I.div_nt0);
@@ -713,17 +713,19 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const CUtensorMa
     int *sJA = reinterpret_cast<int *>(sJraw);
     float *sJT = reinterpret_cast<float *>(sJA + 4 * jv4);
 
-    if (tid == 0) {
-        mbar_init(&bar, 1);
-        const CUtensorMap *tm = tmaps + 6 * fpar;
-        if (!PARTS)  // (a launch of one instance has them among its parameters)
-            for (int c = 0; c < 6; ++c) tmap_acquire(tm + c);
-        mbar_expect_tx(&bar, 6u * (uint32_t)box_bytes);
-        const int x = T0[0] + I.box_lo[0] + I.gh[0];
-        const int y = T0[1] + I.box_lo[1] + I.gh[1];
-        const int z = T0[2] + I.box_lo[2] + I.gh[2];
-        for (int c = 0; c < 6; ++c)
-            tma_load_3d(sbase + c * box_stride, tm + c, x, y, z, &bar);
+    if (warp == 0) {
+        if (lane == 0) {
+            mbar_init(&bar, 1);
+            mbar_expect_tx(&bar, 6u * (uint32_t)box_bytes);
+        }
+        __syncwarp();
+        if (lane < 6) {  // a lane per component: the fences and copies do not wait for one another
+            const CUtensorMap *tm = tmaps + 6 * fpar + lane;
+            if (!PARTS) tmap_acquire(tm);  // (a launch of one instance has them among its parameters)
+            tma_load_3d(sbase + lane * box_stride, tm, T0[0] + I.box_lo[0] + I.gh[0], T0[1] + I.box_lo[1] + I.gh[1],
+                        T0[2] + I.box_lo[2] + I.gh[2], &bar);
+        }
+        __syncwarp();
     }
     if constexpr (kFixed)
         for (int e = tid; e < 2 * jv4; e += kNT)  // A and T
