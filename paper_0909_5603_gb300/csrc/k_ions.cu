@@ -13,11 +13,13 @@
 
 namespace pic {
 
-// This step's ion current on the Jz faces of each instance (one CTA per instance).
+// This step's ion current on the Jz faces of each instance (blockIdx.x), 64 planes a block:
+// the FP64 chain of a plane is long, so each plane has a thread of its own (1024 planes on
+// one block of 256: 13 us).
 template <typename R>
-__global__ void __launch_bounds__(256) k_ion_faces(Launch L)
+__global__ void __launch_bounds__(64) k_ion_faces(Launch L)
 {
-    ion_faces_of<R>(L.inst[blockIdx.x], threadIdx.x, blockDim.x);
+    ion_faces_of<R>(L.inst[blockIdx.x], blockIdx.y * 64 + threadIdx.x, gridDim.y * 64);
 }
 
 // J at the start of a step of a batch: Jx = Jy = 0 and Jz = the ion current of its plane in
@@ -89,25 +91,26 @@ __global__ void __launch_bounds__(256) k_j_init_one(const __grid_constant__ Inst
     }
 }
 
-cudaError_t launch_j_init_one(int fp64, const Launch &L, const InstDev &h, cudaStream_t s)
+cudaError_t launch_ion_faces(int fp64, const Launch &L, int planes, cudaStream_t s)
 {
-    if (h.ion) {
-        if (fp64) k_ion_faces<double><<<1, 256, 0, s>>>(L);
-        else k_ion_faces<float><<<1, 256, 0, s>>>(L);
-    }
+    const int parts = (planes + 63) / 64;
+    const dim3 grid((unsigned)L.ninst, (unsigned)(parts < 1024 ? parts : 1024));
+    if (fp64) k_ion_faces<double><<<grid, 64, 0, s>>>(L);
+    else k_ion_faces<float><<<grid, 64, 0, s>>>(L);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_j_init_one(int fp64, const InstDev &h, cudaStream_t s)
+{
     const unsigned blocks = (unsigned)(((long long)h.P[1] * h.P[2] + 7) / 8);
     if (fp64) k_j_init_one<double><<<blocks, 256, 0, s>>>(h);
     else k_j_init_one<float><<<blocks, 256, 0, s>>>(h);
     return cudaGetLastError();
 }
 
-cudaError_t launch_j_init_batch(int fp64, const Launch &L, bool ions, cudaStream_t s)
+cudaError_t launch_j_init_batch(int fp64, const Launch &L, cudaStream_t s)
 {
     const unsigned blocks = (unsigned)((L.total_cells + 255) / 256);
-    if (ions) {
-        if (fp64) k_ion_faces<double><<<L.ninst, 256, 0, s>>>(L);
-        else k_ion_faces<float><<<L.ninst, 256, 0, s>>>(L);
-    }
     if (fp64) k_j_init_batch<double><<<blocks, 256, 0, s>>>(L);
     else k_j_init_batch<float><<<blocks, 256, 0, s>>>(L);
     return cudaGetLastError();

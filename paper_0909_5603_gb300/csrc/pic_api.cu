@@ -1264,15 +1264,22 @@ static pic_status enqueue_step(pic_ctx *c, int mask)
     int launches = 0;
     if (mask & PIC_PHASE_PARTICLES) {
         tm.begin(4);
+        bool ions = c->h.ion != 0;
+        int planes = c->n[2];
         if (c->is_batch) {
-            bool ions = false;
-            for (auto m : c->members) ions = ions || m->h.ion != 0;
-            CUDA_OR_FAIL(c, launch_j_init_batch(fp64, L, ions, c->stream));
-            launches += ions ? 2 : 1;
-        } else {
-            CUDA_OR_FAIL(c, launch_j_init_one(fp64, L, c->h, c->stream));
-            launches += c->h.ion ? 2 : 1;
+            ions = false;
+            for (auto m : c->members) {
+                ions = ions || m->h.ion != 0;
+                planes = std::max(planes, m->n[2]);
+            }
         }
+        if (ions) {
+            CUDA_OR_FAIL(c, launch_ion_faces(fp64, L, planes, c->stream));
+            launches += 1;
+        }
+        if (c->is_batch) CUDA_OR_FAIL(c, launch_j_init_batch(fp64, L, c->stream));
+        else CUDA_OR_FAIL(c, launch_j_init_one(fp64, c->h, c->stream));
+        launches += 1;
         tm.end(4);
         tm.begin(1);
         CUDA_OR_FAIL(c, launch_scan(L, 0, nullptr, c->stream));

@@ -1,6 +1,7 @@
 """The fused Yee update over its tiles and z chunks, against the FP64 oracle (1e-12, full
 steps, so that the gather reads the periodic images the update stores in the ghost layers):
-grids below, at and just above a tile (32 x 8 columns in 3D, 64 in 2D3V) and a ghost width
+grids below, at and just above what a block puts out (29 x 13 columns in 3D, strips of 29 in
+2D3V) and a ghost width
 (cells that are images beyond both faces of a periodic axis), mixed boundaries, alone and
 as members of a batch."""
 import numpy as np
@@ -16,8 +17,9 @@ FIELDS = [pic.PIC_EX, pic.PIC_EY, pic.PIC_EZ, pic.PIC_BX, pic.PIC_BY, pic.PIC_BZ
 DT = 0.45
 GRIDS = {
     3: [((8, 8, 8), (0, 0, 0)), ((8, 24, 33), (0, 0, 0)), ((33, 9, 26), (0, 1, 0)), ((64, 8, 40), (1, 0, 1)),
-        ((31, 25, 70), (0, 0, 1))],
-    2: [((16, 1, 16), (0, 0, 0)), ((64, 1, 49), (0, 0, 0)), ((65, 1, 130), (0, 0, 1)), ((130, 1, 48), (1, 0, 0))],
+        ((31, 25, 70), (0, 0, 1)), ((29, 13, 24), (1, 1, 0)), ((30, 14, 24), (1, 0, 0)), ((58, 27, 9), (0, 0, 1))],
+    2: [((16, 1, 16), (0, 0, 0)), ((64, 1, 49), (0, 0, 0)), ((65, 1, 130), (0, 0, 1)), ((130, 1, 48), (1, 0, 0)), ((29, 1, 48), (1, 0, 0)),
+        ((59, 1, 50), (0, 0, 0))],
 }
 
 
