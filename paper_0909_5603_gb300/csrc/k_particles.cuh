@@ -1,11 +1,12 @@
 // k_particles.cuh -- the particle half of the boosted-frame PIC step on sm_103a.
 //
-// One CTA per particle tile.  It stages the tile's E and B plus guard cells into shared
-// memory with TMA bulk-tensor copies, loads the tile's particles from the previous
+// One CTA per particle tile, or per part of a crowded one.  It stages the tile's E and B plus
+// guard cells into shared memory with TMA bulk-tensor copies, loads the tile's particles from the previous
 // step's layout (the moved-in sub-ranges of the 27 neighbouring tiles), and for each
 // particle: gathers E, B (shape order 1 or 2, each component at its Yee position), pushes
 // u with the Vay (or Boris) pusher (Sec. 2 of the paper), moves it, and deposits the
-// charge-conserving Esirkepov current into a shared-memory J tile.  Each chunk of
+// charge-conserving Esirkepov current, in FP32 mode into a shared-memory J tile, in FP64 mode
+// with reductions straight to global memory.  Each chunk of
 // particles is written out stably partitioned by the tile it moved to, so the next
 // step finds every tile's particles in contiguous sub-ranges: the array stays sorted
 // by tile at every step with no separate sort pass.  The J tile is flushed to global
