@@ -92,6 +92,117 @@ __global__ void __launch_bounds__(256) k_bhalf(Launch L, int damp)
     Bz[p] = bz;
 }
 
+// The low-dispersion half step of one 3D instance: a thread per column marches along z
+// through tz planes (blockIdx.y) with its 3 x 3 neighbourhood of E on three planes in
+// registers, so that a cell costs 27 loads of E instead of the 108 that k_bhalf's six
+// differences ask for, which bound it there (addresses and L1, at 23 % of HBM).  The
+// differences and their order are k_bhalf's.  128 registers, no spills, 16 warps an SM, and
+// bound by the latency of a plane's loads; the three updates of a step: 64x64x512 162 -> 112
+// us, 128x128x512 620 -> 395, 32x32x256 38 -> 33.  (Unrolled by three planes, so that none is
+// moved: 140 us; with 96 registers 127.)
+template <typename R>
+__device__ __forceinline__ R ck_sum(const R d[9])
+{
+    R sum = R(0);
+#pragma unroll
+    for (int m = 0; m < 9; ++m) {
+        const int edges = (m / 3 != 1) + (m % 3 != 1);
+        const R w = edges == 0 ? R(7.0 / 12.0) : (edges == 1 ? R(1.0 / 12.0) : R(1.0 / 48.0));
+        sum += w * d[m];
+    }
+    return sum;
+}
+
+// differences of the neighbourhood f[z][y][x] (entry 1 the cell itself), averaged as ck_diff
+// does: its outer loop runs over axis a + 1, its inner one over axis a + 2
+template <typename R, int A>
+__device__ __forceinline__ R ck_diff3(const R (&f)[3][3][3])
+{
+    R d[9];
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            d[3 * b + c] = A == 0 ? f[c][b][2] - f[c][b][1] : (A == 1 ? f[b][2][c] - f[b][1][c] : f[2][c][b] - f[1][c][b]);
+    return ck_sum(d);
+}
+
+__global__ void __launch_bounds__(128) k_bhalf_ck3(Launch L, int damp, int tz)
+{
+    using R = float;
+    const InstDev &I = L.inst[0];
+    const int n0 = I.n[0], n1 = I.n[1], n2 = I.n[2];
+    const int col = blockIdx.x * 128 + threadIdx.x;
+    if (col >= n0 * n1) return;
+    CellPos c;
+    c.ii = 0;
+    c.j = fast_div(col, I.div_n0);
+    c.i = col - c.j * n0;
+    const EBPtr F = cur_eb(I);
+    const StepCoef<R> &K = coef<R>(I);
+    const R h = K.half_dt;
+    const R ix = K.inv_dx[0], iy = K.inv_dx[1], iz = K.inv_dx[2];
+    const long long sz = I.sz, base = (c.i + I.gh[0]) + I.sy * (c.j + I.gh[1]) + sz * I.gh[2];
+    int off[3][3];  // of the neighbours in a plane, [y][x]
+    {
+        const int ox[3] = {I.bc[0] == 0 && c.i == 0 ? n0 - 1 : -1, 0, I.bc[0] == 0 && c.i == n0 - 1 ? 1 - n0 : 1};
+        const int ny = n1 - 1, sy = (int)I.sy;
+        const int oy[3] = {I.bc[1] == 0 && c.j == 0 ? ny * sy : -sy, 0, I.bc[1] == 0 && c.j == ny ? -ny * sy : sy};
+#pragma unroll
+        for (int y = 0; y < 3; ++y)
+#pragma unroll
+            for (int x = 0; x < 3; ++x) off[y][x] = oy[y] + ox[x];
+    }
+    const bool perz = I.bc[2] == 0;
+    const R *const E[3] = {(const R *)F.E[0] + base, (const R *)F.E[1] + base, (const R *)F.E[2] + base};
+    R *const B[3] = {(R *)F.B[0] + base, (R *)F.B[1] + base, (R *)F.B[2] + base};
+    R f[3][3][3][3];  // [component][plane][y][x]
+    auto load = [&](int k, int z) {
+        const long long o = sz * (perz ? (k < 0 ? n2 - 1 : (k == n2 ? 0 : k)) : k);
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+#pragma unroll
+            for (int y = 0; y < 3; ++y)
+#pragma unroll
+                for (int x = 0; x < 3; ++x) f[m][z][y][x] = __ldg(E[m] + o + off[y][x]);
+    };
+    const int k0 = blockIdx.y * tz, k1 = min(k0 + tz, n2);
+    load(k0 - 1, 0);
+    load(k0, 1);
+    for (c.k = k0; c.k < k1; ++c.k) {
+        const long long o = sz * c.k;
+        load(c.k + 1, 2);
+        const R b0 = B[0][o], b1 = B[1][o], b2 = B[2][o];
+        const R dEy_dz = ck_diff3<R, 2>(f[1]) * iz;
+        const R dEx_dz = ck_diff3<R, 2>(f[0]) * iz;
+        const R dEz_dx = ck_diff3<R, 0>(f[2]) * ix;
+        const R dEy_dx = ck_diff3<R, 0>(f[1]) * ix;
+        const R dEz_dy = ck_diff3<R, 1>(f[2]) * iy;
+        const R dEx_dy = ck_diff3<R, 1>(f[0]) * iy;
+        R bx = b0 - h * (dEz_dy - dEy_dz);
+        R by = b1 - h * (dEx_dz - dEz_dx);
+        R bz = b2 - h * (dEy_dx - dEx_dy);
+        if (damp) {
+            const R d = damp_factor<R>(I, c);
+            bx *= d;
+            by *= d;
+            bz *= d;
+        }
+        B[0][o] = bx;
+        B[1][o] = by;
+        B[2][o] = bz;
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+#pragma unroll
+            for (int y = 0; y < 3; ++y)
+#pragma unroll
+                for (int x = 0; x < 3; ++x) {
+                    f[m][0][y][x] = f[m][1][y][x];
+                    f[m][1][y][x] = f[m][2][y][x];
+                }
+    }
+}
+
 // The fused Yee update (maxwell_fused_block).  The CTA of an
 // instance that finishes last switches it to the buffer pair it wrote (every CTA has read
 // the parity by then), so that no launch follows for it.
@@ -457,34 +568,43 @@ cudaError_t launch_filter(int fp64, const Launch &L, const long long *const penc
     return cudaGetLastError();
 }
 
-template <typename R, bool CK>
-static void maxwell_kernels(const Launch &L, int filtered, unsigned nb, cudaStream_t s)
-{
-    k_bhalf<R, CK><<<nb, 256, 0, s>>>(L, 0);
-    k_efull<R><<<nb, 256, 0, s>>>(L, filtered);
-    k_bhalf<R, CK><<<nb, 256, 0, s>>>(L, 1);
-}
-
-cudaError_t launch_maxwell(int fp64, int solver, const Launch &L, int filtered, cudaStream_t s)
+// One half step of B.  ck_n: the cells of a launch of one 3D instance under the
+// low-dispersion solver, else null.  The FP32 march takes chunks of about 32 planes or, on
+// smaller grids, as many as fill the 608 resident blocks once (a chunk loads two planes more
+// than it puts out; 64x64x512: 8 blocks an SM 115, 4 blocks 112 us for the three updates).
+// In FP64 the per-cell kernel stays: both are bound by the FP64 pipe (64x64x512: 1108 us,
+// the march 1126).
+template <typename R>
+static void bhalf(int solver, const Launch &L, const int *ck_n, int damp, cudaStream_t s)
 {
     const unsigned nb = blocks_for(L.total_cells, 256);
-    const bool ck = solver == PIC_SOLVER_CK;
+    if (solver == PIC_SOLVER_CK && ck_n) {
+        const long long cols = blocks_for((long long)ck_n[0] * ck_n[1], 128);
+        const long long waves = (cols * ((ck_n[2] + 31) / 32) + 607) / 608;
+        const int chunks = (int)std::max(1LL, std::min(608 * waves / cols, 65535LL));
+        const int tz = (ck_n[2] + chunks - 1) / chunks;
+        k_bhalf_ck3<<<dim3((unsigned)cols, (ck_n[2] + tz - 1) / tz), 128, 0, s>>>(L, damp, tz);
+    } else if (solver == PIC_SOLVER_CK) {
+        k_bhalf<R, true><<<nb, 256, 0, s>>>(L, damp);
+    } else {
+        k_bhalf<R, false><<<nb, 256, 0, s>>>(L, damp);
+    }
+}
+
+cudaError_t launch_bhalf(int fp64, int solver, const Launch &L, const int *ck_n, int damp, cudaStream_t s)
+{
     if (fp64)
-        ck ? maxwell_kernels<double, true>(L, filtered, nb, s) : maxwell_kernels<double, false>(L, filtered, nb, s);
+        bhalf<double>(solver, L, nullptr, damp, s);
     else
-        ck ? maxwell_kernels<float, true>(L, filtered, nb, s) : maxwell_kernels<float, false>(L, filtered, nb, s);
+        bhalf<float>(solver, L, ck_n, damp, s);
     return cudaGetLastError();
 }
 
-cudaError_t launch_bhalf(int fp64, int solver, const Launch &L, int damp, cudaStream_t s)
+cudaError_t launch_maxwell(int fp64, int solver, const Launch &L, const int *ck_n, int filtered, cudaStream_t s)
 {
-    const unsigned nb = blocks_for(L.total_cells, 256);
-    const bool ck = solver == PIC_SOLVER_CK;
-    if (fp64)
-        ck ? k_bhalf<double, true><<<nb, 256, 0, s>>>(L, damp) : k_bhalf<double, false><<<nb, 256, 0, s>>>(L, damp);
-    else
-        ck ? k_bhalf<float, true><<<nb, 256, 0, s>>>(L, damp) : k_bhalf<float, false><<<nb, 256, 0, s>>>(L, damp);
-    return cudaGetLastError();
+    cudaError_t e = launch_bhalf(fp64, solver, L, ck_n, 0, s);
+    if (e == cudaSuccess) e = launch_efull(fp64, L, filtered, s);
+    return e == cudaSuccess ? launch_bhalf(fp64, solver, L, ck_n, 1, s) : e;
 }
 
 cudaError_t launch_efull(int fp64, const Launch &L, int filtered, cudaStream_t s)

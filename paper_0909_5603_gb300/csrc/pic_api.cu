@@ -1318,6 +1318,7 @@ static pic_status enqueue_step(pic_ctx *c, int mask)
         if (c->ant_on) ants.push_back(c);
         for (auto m : c->members)
             if (m->ant_on) ants.push_back(m);
+        const int *ck_n = c->opt.solver == PIC_SOLVER_CK && !c->is_batch && c->ndim == 3 ? c->n : nullptr;
         if (ants.empty() && c->opt.solver == PIC_SOLVER_YEE && c->pencil_total[3] > 0) {
             // the fused update, with the buffer switch and the periodic images
             const int nin = c->is_batch ? (int)c->members.size() : 1;
@@ -1326,12 +1327,12 @@ static pic_status enqueue_step(pic_ctx *c, int mask)
             launches += 1;
             fused = true;
         } else if (ants.empty()) {
-            CUDA_OR_FAIL(c, launch_maxwell(fp64, c->opt.solver, L, filtered, c->stream));
+            CUDA_OR_FAIL(c, launch_maxwell(fp64, c->opt.solver, L, ck_n, filtered, c->stream));
             launches += 3;
         } else {
             // the antenna's boundary terms and lattice steps between the Yee sub-updates
             cudaStream_t s = c->stream;
-            CUDA_OR_FAIL(c, launch_bhalf(fp64, c->opt.solver, L, 0, s));
+            CUDA_OR_FAIL(c, launch_bhalf(fp64, c->opt.solver, L, ck_n, 0, s));
             for (auto m : ants) {
                 CUDA_OR_FAIL(c, launch_ant_bterm(fp64, c->opt.solver == PIC_SOLVER_CK, m->d_inst, m->h, m->ant, 0, s));
                 CUDA_OR_FAIL(c, launch_ant_lattice(m->ant, m->dt, m->dx[2], 0, s));
@@ -1341,7 +1342,7 @@ static pic_status enqueue_step(pic_ctx *c, int mask)
                 CUDA_OR_FAIL(c, launch_ant_eterm(fp64, m->d_inst, m->h, m->ant, s));
                 CUDA_OR_FAIL(c, launch_ant_lattice(m->ant, m->dt, m->dx[2], 1, s));
             }
-            CUDA_OR_FAIL(c, launch_bhalf(fp64, c->opt.solver, L, 1, s));
+            CUDA_OR_FAIL(c, launch_bhalf(fp64, c->opt.solver, L, ck_n, 1, s));
             for (auto m : ants) {
                 CUDA_OR_FAIL(c, launch_ant_bterm(fp64, c->opt.solver == PIC_SOLVER_CK, m->d_inst, m->h, m->ant, 1, s));
                 CUDA_OR_FAIL(c, launch_ant_lattice(m->ant, m->dt, m->dx[2], 2, s));

@@ -192,9 +192,10 @@ inline long long filter_pencils(const int n[3], int ndim, int axis)
     if (axis == 1) return cols * ((n[1] + kP - 1) / kP) * n[2];
     return cols * ((n[2] + kP - 1) / kP) * n[1];
 }
-cudaError_t launch_maxwell(int fp64, int solver, const Launch &L, int filtered, cudaStream_t s);
+// ck_n: the cells of a launch of one 3D instance under the low-dispersion solver, else null
+cudaError_t launch_maxwell(int fp64, int solver, const Launch &L, const int *ck_n, int filtered, cudaStream_t s);
 // the three sub-updates of launch_maxwell, for interleaving the antenna's kernels
-cudaError_t launch_bhalf(int fp64, int solver, const Launch &L, int damp, cudaStream_t s);
+cudaError_t launch_bhalf(int fp64, int solver, const Launch &L, const int *ck_n, int damp, cudaStream_t s);
 cudaError_t launch_efull(int fp64, const Launch &L, int filtered, cudaStream_t s);
 // antenna: what = 0 adds the incident field downstream of the plane (when set), 1 the
 // values the plane passed in the last phase; B_y / E_x terms of the boundary; 1D lattice
