@@ -40,7 +40,7 @@ struct SrcTable {
     int k0[kDirs];              // its first chunk with particles of the slots asked for
     int chpre[kDirs + 1];       // prefix of the chunks from k0 on that may hold such particles
     int nsub;                   // non-empty (source, chunk) sub-ranges, -1 if > kMaxSub
-    int sub_slot[kMaxSub + 1];  // first destination slot of each sub-range, then their end
+    int sub_slot[kMaxSub + 1];  // first destination slot of each sub-range, then kSlotEnd
     int sub_pos[kMaxSub];       // buffer position of each sub-range's first particle
     int warp_tmp[32];
 };
@@ -234,7 +234,7 @@ static __device__ void build_sources(const InstDev &I, int lay, int tx, int ty, 
     if (tid == 0) {
         const bool fits = written <= kMaxSub;
         S.nsub = fits ? written : -1;
-        if (fits) S.sub_slot[written] = min(s1, S.count);
+        if (fits) S.sub_slot[written] = kSlotEnd;
     }
     __syncthreads();
 }
@@ -266,23 +266,19 @@ __device__ __forceinline__ int slot_position(const InstDev &I, int lay, const Sr
 }
 
 // Buffer position of slot p (-1 without a particle) for the lanes of a warp at consecutive
-// slots from p0 on.  With at most 64 sub-ranges the one of p0 is found by the warp together
+// slots from p0 on.  With 1 to 64 sub-ranges the one of p0 is found by the warp together
 // (two votes) and each lane walks on from there, a step or two: sub-ranges are tens of
 // slots long.  Called by the whole warp.
 __device__ __forceinline__ int slot_position_warp(const InstDev &I, int lay, const SrcTable &S, int p0, int p, bool live,
                                                   int lane)
 {
-    if ((unsigned)S.nsub > 64u) return live ? slot_position(I, lay, S, p) : -1;
+    if ((unsigned)(S.nsub - 1) >= 64u) return live ? slot_position(I, lay, S, p) : -1;
     const int n = S.nsub;
     const unsigned v0 = __ballot_sync(0xffffffffu, lane < n && S.sub_slot[lane] <= p0);
     const unsigned v1 = __ballot_sync(0xffffffffu, lane + 32 < n && S.sub_slot[lane + 32] <= p0);
     if (!live) return -1;
-    int e = __popc(v0) + __popc(v1) - 1;
-    int at = S.sub_slot[e];
-    for (int next = S.sub_slot[e + 1]; next <= p; next = S.sub_slot[e + 1]) {  // (ends at sub_slot[n] > p)
-        ++e;
-        at = next;
-    }
+    int at;
+    const int e = sub_range_from(S.sub_slot, __popc(v0) + __popc(v1) - 1, p, at);
     return S.sub_pos[e] + (p - at);
 }
 
@@ -504,7 +500,7 @@ __device__ __forceinline__ void tile_sources_warp(const Launch &L, int g, SrcScr
     if (lane == 0) {
         rec[0] = slot_run;
         rec[1] = fits ? written : -1;
-        if (fits) rec[kRecSlot + written] = slot_run;
+        if (fits) rec[kRecSlot + written] = kSlotEnd;
         // the parts of the coming phase (the scan has laid out its output)
         const int *cb = I.chunk_base[1 - lay];
         const int ch = cb[t + 1] - cb[t], m = part_chunks(cb[I.ntiles], I.part_min);

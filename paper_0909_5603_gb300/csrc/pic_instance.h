@@ -54,6 +54,26 @@ __host__ __device__ __forceinline__ int readout_window(int cap)
     return w > 8192 ? w : 8192;
 }
 
+// The sub-range of slot p in a source table of at least one (sub_slot: their first slots,
+// ascending, then kSlotEnd), walking on from sub-range e, the last one known to start at or
+// before p; `at` is its first slot.  The end stops the walk at any p: where a tile's
+// population and its source records disagree (a recorded device error: an earlier launch
+// left the layout half written) p can lie beyond the slots that the table holds, and with the
+// slot after the last one for its end the walk would read on through the rest of the block's
+// shared memory.  (An end that stops it costs no instruction: the particle phase of the
+// 128x128x1024 stage stays at 4.03 ms.)
+constexpr int kSlotEnd = INT_MAX;
+__host__ __device__ __forceinline__ int sub_range_from(const int *sub_slot, int e, int p, int &at)
+{
+    e = e > 0 ? e : 0;  // (no sub-range starts at or before p)
+    at = sub_slot[e];
+    for (int next = sub_slot[e + 1]; next <= p; next = sub_slot[e + 1]) {
+        ++e;
+        at = next;
+    }
+    return e;
+}
+
 // Division of 0 <= x < 2^31 by a fixed divisor d >= 1 without a divide instruction
 // (Granlund & Montgomery, "Division by invariant integers using multiplication", 1994,
 // round-up variant): s = ceil(log2 d), m = floor(2^(32+s) / d) + 1 (33 bits), then
