@@ -257,12 +257,14 @@ pic_status pic_run_phases(pic_ctx *ctx, int phase_mask);
  * staggered layout above.  J is the current used by the last Maxwell update (after the
  * filter).  PIC_RHO deposits the particles' charge with their shape (plus the ion
  * background) into per-context FP64 memory; PIC_DIVE is the node divergence of E.
- * Synchronises; PIC_ERR_ARG for an unknown component or a short buffer. */
+ * Synchronises; PIC_ERR_ARG for an unknown component or a short buffer.  After an earlier
+ * step's device error (pic_synchronize) that error is returned, host_out untouched. */
 pic_status pic_get_field(pic_ctx *ctx, int comp, double *host_out, size_t count);
 
 /* Copies ncomp components (as for pic_get_field, Sec. 2) into
  * host_out[ncomp][n2][n1][n0], count >= ncomp n0 n1 n2; comps[i] as pic_get_field.
- * Synchronises; PIC_ERR_ARG for an unknown component, ncomp < 1 or a short buffer. */
+ * Synchronises; PIC_ERR_ARG for an unknown component, ncomp < 1 or a short buffer; errors
+ * as for pic_get_field. */
 pic_status pic_get_fields(pic_ctx *ctx, const int *comps, int ncomp, double *host_out, size_t count);
 
 /* Gauss-law residual on the nodes: *max_abs = max |div E - rho| and, when rms is not NULL,

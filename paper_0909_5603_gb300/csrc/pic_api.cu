@@ -1510,22 +1510,18 @@ extern "C" pic_status pic_synchronize(pic_ctx *ctx)
 // ------------------------------------------------------------------------------------
 // getters
 // ------------------------------------------------------------------------------------
-// Components one after the other through the dense scratch into host_out, queued on the
-// stream behind the work in flight with one synchronisation at the end (six components of
-// a 128x128 grid: 320 us with three synchronisations each).  The density walks the
-// particle layout, which a step that ended in a device error may have left half written:
-// such an error is looked for first.
+// Components one after the other through the dense scratch into host_out.  The device error
+// word is read first, behind the work in flight: a call that reports an error leaves
+// host_out as it was (and the density walks the particle layout, which a step that ended in
+// one may have left half written).  The components are then queued with one synchronisation
+// at the end (six components of a 64x64 grid: 110 us, with three synchronisations each 247).
 static pic_status read_fields(pic_ctx *c, const int *comps, int ncomp, double *host_out)
 {
     const size_t bytes = sizeof(double) * (size_t)c->ncell;
     cudaStream_t s = c->stream;
     cudaSetDevice(c->device);
-    for (int i = 0; i < ncomp; ++i)
-        if (comps[i] == PIC_RHO) {
-            const pic_status st = pic_synchronize(c);
-            if (st != PIC_OK) return st;
-            break;
-        }
+    const pic_status st = check_device_error(c);
+    if (st != PIC_OK) return st;
     for (int i = 0; i < ncomp; ++i) {
         if (comps[i] == PIC_RHO) {
             CUDA_OR_FAIL(c, cudaMemsetAsync(c->d_dense, 0, bytes, s));
@@ -1537,11 +1533,9 @@ static pic_status read_fields(pic_ctx *c, const int *comps, int ncomp, double *h
         }
         CUDA_OR_FAIL(c, cudaMemcpyAsync(host_out + (size_t)i * c->ncell, c->d_dense, bytes, cudaMemcpyDeviceToHost, s));
     }
-    int err = 0;
-    CUDA_OR_FAIL(c, cudaMemcpyAsync(&err, c->h.err, sizeof(int), cudaMemcpyDeviceToHost, s));
     CUDA_OR_FAIL(c, cudaStreamSynchronize(s));
     CUDA_OR_FAIL(c, cudaGetLastError());
-    return device_error_status(c, err);
+    return PIC_OK;
 }
 
 extern "C" pic_status pic_get_field(pic_ctx *ctx, int comp, double *host_out, size_t count)
