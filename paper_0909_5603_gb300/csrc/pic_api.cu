@@ -1522,18 +1522,22 @@ static pic_status read_fields(pic_ctx *c, const int *comps, int ncomp, double *h
     cudaSetDevice(c->device);
     const pic_status st = check_device_error(c);
     if (st != PIC_OK) return st;
-    for (int i = 0; i < ncomp; ++i) {
+    auto queue = [&](int i) {
+        cudaError_t e;
         if (comps[i] == PIC_RHO) {
-            CUDA_OR_FAIL(c, cudaMemsetAsync(c->d_dense, 0, bytes, s));
-            if (c->loaded) CUDA_OR_FAIL(c, launch_rho(c->order, c->fp64, c->L, c->h, c->d_dense, s));
+            e = cudaMemsetAsync(c->d_dense, 0, bytes, s);
+            if (e == cudaSuccess && c->loaded) e = launch_rho(c->order, c->fp64, c->L, c->h, c->d_dense, s);
         } else if (comps[i] == PIC_DIVE) {
-            CUDA_OR_FAIL(c, launch_dive(c->fp64, c->h, c->d_dense, c->ncell, s));
+            e = launch_dive(c->fp64, c->h, c->d_dense, c->ncell, s);
         } else {
-            CUDA_OR_FAIL(c, launch_pack(c->fp64, c->h, comps[i], c->last_filtered, c->d_dense, c->ncell, s));
+            e = launch_pack(c->fp64, c->h, comps[i], c->last_filtered, c->d_dense, c->ncell, s);
         }
-        CUDA_OR_FAIL(c, cudaMemcpyAsync(host_out + (size_t)i * c->ncell, c->d_dense, bytes, cudaMemcpyDeviceToHost, s));
-    }
-    CUDA_OR_FAIL(c, cudaStreamSynchronize(s));
+        return e == cudaSuccess
+                   ? cudaMemcpyAsync(host_out + (size_t)i * c->ncell, c->d_dense, bytes, cudaMemcpyDeviceToHost, s)
+                   : e;
+    };
+    const cudaError_t e = queue_then_wait(ncomp, queue, [&] { return cudaStreamSynchronize(s); });
+    if (e != cudaSuccess) return fail(c, PIC_ERR_CUDA, "field read-out failed: %s", cudaGetErrorString(e));
     CUDA_OR_FAIL(c, cudaGetLastError());
     return PIC_OK;
 }

@@ -225,6 +225,18 @@ cudaError_t launch_dive(int fp64, const InstDev &I, double *dense, long long nce
 cudaError_t launch_residual(const double *a, const double *b, long long n, unsigned long long *max_bits, double *sumsq,
                             cudaStream_t s);
 
+// Queues items 0 .. n - 1 of work that writes to the caller's memory, up to the first that
+// cannot be queued, and waits for what was queued in either case: when an error is returned,
+// no copy into that memory is still running.  Returns the first error.
+template <typename Queue, typename Wait>
+cudaError_t queue_then_wait(int n, Queue queue, Wait wait)
+{
+    cudaError_t first = cudaSuccess;
+    for (int i = 0; i < n && first == cudaSuccess; ++i) first = queue(i);
+    const cudaError_t waited = wait();
+    return first != cudaSuccess ? first : waited;
+}
+
 // Read-only view of a pic_ctx (defined in pic_api.cu) for entry points in other files.
 struct CtxView {
     const Launch *launch;
