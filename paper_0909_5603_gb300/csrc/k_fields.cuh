@@ -396,6 +396,15 @@ __device__ __forceinline__ int filter_source(int &q, int n, int P, bool per)
     return -1;
 }
 
+// v, negated when neg.  FP64: in the sign bit, as the FP64 pipe, which a select between v and
+// -v goes through, bounds the filter there (64x64x128 periodic cells, one pass: 58 us
+// with the select, 53 without any).
+__device__ __forceinline__ float negate_if(float v, bool neg) { return neg ? -v : v; }
+__device__ __forceinline__ double negate_if(double v, bool neg)
+{
+    return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000 : 0), __double2loint(v));
+}
+
 // y and z axes: lane = x column (coalesced), each warp takes kPencil / 8 consecutive
 // cells along the axis and loads them with P halo cells per side into registers
 // (filter_source); the outputs are (2P+1)-tap convolutions.  Four blocks of 64 registers per
@@ -456,7 +465,7 @@ __device__ __forceinline__ void filter_col_block(const Launch &L, int axis, cons
             for (int comp = 0; comp < 3; ++comp)
 #pragma unroll
                 for (int m = 0; m < W; ++m)
-                    if ((neg >> m) & 1u) win[comp][m] = -win[comp][m];
+                    win[comp][m] = negate_if(win[comp][m], (neg >> m) & 1u);
         }
     }
 #pragma unroll
@@ -536,7 +545,7 @@ __device__ __forceinline__ void filter_row_block(const Launch &L, const long lon
         for (int comp = 0; comp < 3; ++comp)
 #pragma unroll
             for (int c = 0; c < NC; ++c)
-                if (32 * c + lane < W) win[comp][32 * c + lane] = qneg[c] ? -pre[j][comp][c] : pre[j][comp][c];
+                if (32 * c + lane < W) win[comp][32 * c + lane] = negate_if(pre[j][comp][c], qneg[c]);
         __syncwarp();
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
