@@ -487,7 +487,7 @@ __device__ __forceinline__ void filter_col_block(const Launch &L, int axis, cons
 // slice of shared memory (warp-synchronous, no block barrier) and each lane forms two
 // outputs from it, convolutions over the window (filter_source).  (With the passes run one
 // by one in the lanes near an absorbing face, beside the convolution of the others, the
-// three axes took 201 us instead of 96 for 48x48x128 FP64 cells, and 382 instead of 324 us
+// three axes took 201 us instead of 89 for 48x48x128 FP64 cells, and 382 instead of 324 us
 // for 128x128x1024 FP32 ones.)
 // sw: shared memory for the windows, 8 x 3 x (kPencil + 2P) values
 template <typename R, int P>
