@@ -575,7 +575,7 @@ cudaError_t launch_filter(int fp64, const Launch &L, const long long *const penc
 // smaller grids, as many as fill the 608 resident blocks once (a chunk loads two planes more
 // than it puts out; 64x64x512: 8 blocks an SM 115, 4 blocks 112 us for the three updates).
 // In FP64 the per-cell kernel stays: both are bound by the FP64 pipe (64x64x512: 1108 us,
-// the march 1126).
+// the march 1126).  2D3V and batches keep it too; no march has been written for them.
 template <typename R>
 static void bhalf(int solver, const Launch &L, const int *ck_n, int damp, cudaStream_t s)
 {

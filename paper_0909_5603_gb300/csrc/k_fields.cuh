@@ -408,7 +408,9 @@ __device__ __forceinline__ double negate_if(double v, bool neg)
 // y and z axes: lane = x column (coalesced), each warp takes kPencil / 8 consecutive
 // cells along the axis and loads them with P halo cells per side into registers
 // (filter_source); the outputs are (2P+1)-tap convolutions.  Four blocks of 64 registers per
-// SM (what the blocks at the faces spill is little) hide the loads better than three of 80.
+// SM in FP32 hide the loads better than three of 80, also with the spills of the blocks at
+// the faces (100 bytes with three passes, 204 with four; all axes of 128x128x256 cells with
+// four passes: 99 us periodic and 99 absorbing, 127 and 137 before).
 template <typename R, int P>
 __device__ __forceinline__ void filter_col_block(const Launch &L, int axis, const long long *pencil_start, int src_is_jt,
                                                  const long long g)

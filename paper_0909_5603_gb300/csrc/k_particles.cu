@@ -310,7 +310,7 @@ cudaError_t launch_readout(int fp64, const Launch &L, int cap, const int *const 
     return cudaGetLastError();
 }
 
-// Blocks of the chunk walks: as many as are resident, fewer when there are fewer chunks.
+// Blocks of the chunk walks: eight for each SM, fewer when there are fewer chunks.
 static unsigned walk_blocks(int chunk_cap)
 {
     return (unsigned)std::max(1, std::min(152 * 8, (chunk_cap + 7) / 8));

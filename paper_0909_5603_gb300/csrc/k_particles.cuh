@@ -1131,7 +1131,7 @@ __device__ __forceinline__ void particle_tile(const InstDev &I, const CUtensorMa
 }
 
 // Blocks per SM that the registers of the particle kernel are bounded for.  The 2D3V body
-// fits 80 registers with 12 bytes of spills (a launch of one instance), so three blocks of
+// fits 80 registers with 4 bytes of spills (order 2; 24 in a batch), so three blocks of
 // 256 threads hide more of one another's waits (a batch of 32 instances: 1.21 -> 1.15 ms); the
 // 3D one would spill 230 bytes, which costs more than the warps give (4.45 against 4.19 ms).
 template <int ND, typename R>

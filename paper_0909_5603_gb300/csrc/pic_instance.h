@@ -30,15 +30,16 @@ constexpr int kSrcRec = (kRecPos + kSubCache + 3) / 4 * 4;  // ints per tile
 // A tile crowded with particles is worked on by several CTAs (parts) of the particle
 // kernel in a launch of one instance.  A part takes part_chunks() chunks; a tile is split
 // when it holds more than twice that.  kMaxOver bounds the parts beyond the first over all
-// tiles: their number is at most total / part_chunks(total) <= kMaxOver = two for each of
-// the 2 x 152 CTAs that are resident, so that the largest part is about half of a CTA's
-// share of the launch: a bunch of 2^20 electrons in 64x64x256 cells, whose fullest tile
-// holds 520 of its 4,500 chunks, is then balanced.  Parts have at least part_min chunks: 8
-// where there are tiles enough for the resident CTAs, as shorter ones would spend more on
-// staging the fields and flushing J than on their particles; 1 where there are not (128x128
-// cells are 64 tiles) and in FP64, where a chunk takes 50 us and its current needs no flush.
+// tiles: their number is at most total / part_chunks(total) <= kMaxOver = four for each of
+// the 152 SMs, which hold two CTAs of the 3D FP32 kernel (three in 2D3V, one in FP64), so
+// that the largest part is about half of such a CTA's share of the launch: a bunch of 2^20
+// electrons in 64x64x256 cells, whose fullest tile holds 520 of its 4,500 chunks, is then
+// balanced.  Parts have at least part_min chunks: 8 in FP32 from kResidentParts tiles on,
+// where shorter ones would spend more on staging the fields and flushing J than on their
+// particles; 1 in smaller grids, whose tiles alone leave SMs idle (128x128 cells are 64
+// tiles), and in FP64, where a chunk takes 50 us and its current needs no flush.
 constexpr int kMaxOver = 608;
-constexpr int kResidentParts = 304;  // 2 CTAs on each of 152 SMs
+constexpr int kResidentParts = 304;  // the CTAs of the 3D FP32 kernel that are resident at once
 
 __host__ __device__ __forceinline__ int part_chunks(int total_chunks, int part_min)
 {
